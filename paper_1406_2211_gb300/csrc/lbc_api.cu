@@ -747,7 +747,11 @@ void enqueue_step(lbc_box* b, cudaStream_t s, int64_t* launches, int phase = 0,
           // them at their force points
           fd = P.drift_setup(first ? 0.5 * dt : 0.0, 0.0, 0.0, true, false, true);
           fd.at_force_point = first ? 0 : 1;
-          fd.pos_out = nullptr;             // the gather writes the next force point
+          // the gather writes the next force point and the kicked velocity,
+          // and uses the intrinsic force itself
+          fd.pos_out = nullptr;
+          fd.vel_out = nullptr;
+          fd.fint_out = nullptr;
         }
         GatherArgs a = P.gather_base();
         if (fused) {

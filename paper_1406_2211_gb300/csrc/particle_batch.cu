@@ -14,6 +14,7 @@
 namespace lbc {
 
 int gather_variant(const PartArgs& p, const GatherArgs& a);
+int gather_lanes(int var);
 
 namespace {
 
@@ -92,12 +93,14 @@ small_sort_batch_kernel(const PartEntry* __restrict__ tab, int n) {
 }
 
 template <typename S, bool WALLS, int ST, int VAR>
-__global__ void __launch_bounds__(GATHER_THREADS, (VAR == GV_LIGHT) ? 6 : 4)
+__global__ void __launch_bounds__(GATHER_THREADS,
+                                  (VAR == GV_LIGHT || VAR == GV_CACHED || VAR == GV_OCT) ? 6 : 4)
 gather_batch_kernel(const PartEntry* __restrict__ tab, int n) {
   __shared__ SharedEntry<HEAD + U_GM> se;
   const PartEntry& e = stage<U_GM>(tab, n, se);
-  gather_body<S, WALLS, ST, VAR>(e.p, e.u.gm.g,
-                                 (blockIdx.x - e.block0) * (long long)blockDim.x + threadIdx.x);
+  const long long gid = (blockIdx.x - e.block0) * (long long)blockDim.x + threadIdx.x;
+  if constexpr (VAR == GV_OCT) gather_oct_body<S, WALLS>(e.p, e.u.gm.g, gid);
+  else gather_body<S, WALLS, ST, VAR>(e.p, e.u.gm.g, gid);
 }
 
 template <int ST>
@@ -135,16 +138,19 @@ void gather_batch_st(int ST, unsigned grid, const PartEntry* tab, int n, cudaStr
   else gather_batch_kernel<S, WALLS, 2, VAR><<<grid, GATHER_THREADS, 0, s>>>(tab, n);
 }
 
+template <typename S, bool WALLS>
+void gather_batch_w(int ST, int var, unsigned grid, const PartEntry* tab, int n, cudaStream_t s) {
+  if (var == GV_OCT) gather_batch_kernel<S, WALLS, 0, GV_OCT><<<grid, GATHER_THREADS, 0, s>>>(tab, n);
+  else if (var == GV_CACHED) gather_batch_st<S, WALLS, GV_CACHED>(ST, grid, tab, n, s);
+  else if (var == GV_LIGHT) gather_batch_st<S, WALLS, GV_LIGHT>(ST, grid, tab, n, s);
+  else gather_batch_st<S, WALLS, GV_FULL>(ST, grid, tab, n, s);
+}
+
 template <typename S>
 void gather_batch_s(bool walls, int ST, int var, unsigned grid, const PartEntry* tab, int n,
                     cudaStream_t s) {
-  if (walls) {
-    if (var == GV_LIGHT) gather_batch_st<S, true, GV_LIGHT>(ST, grid, tab, n, s);
-    else gather_batch_st<S, true, GV_FULL>(ST, grid, tab, n, s);
-  } else {
-    if (var == GV_LIGHT) gather_batch_st<S, false, GV_LIGHT>(ST, grid, tab, n, s);
-    else gather_batch_st<S, false, GV_FULL>(ST, grid, tab, n, s);
-  }
+  if (walls) gather_batch_w<S, true>(ST, var, grid, tab, n, s);
+  else gather_batch_w<S, false>(ST, var, grid, tab, n, s);
 }
 
 template <typename S>
@@ -184,8 +190,10 @@ int part_op_blocks(int kind, const PartEntry& e) {
   const long long M = e.p.M;
   switch (kind) {
     case OP_DRIFT:
-    case OP_GATHER:
       return (int)((M + GATHER_THREADS - 1) / GATHER_THREADS);
+    case OP_GATHER:
+      return (int)((gather_lanes(gather_variant(e.p, e.u.gm.g)) * M + GATHER_THREADS - 1) /
+                   GATHER_THREADS);
     case OP_SMALL_SORT:
       return 1;
     case OP_SPREAD: {

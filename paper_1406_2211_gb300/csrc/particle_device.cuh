@@ -276,6 +276,8 @@ __device__ inline bool near_home_f(const Geom& g, uint32_t home, const double (&
 }
 
 // ------------------------------------------------------------ drift / forces
+constexpr int BONDS_AT_ONCE = 2;
+
 // One marker's sub-step (see DriftArgs): writes its new position, velocity,
 // intrinsic force and key, and returns the position, velocity and force.
 template <typename C>
@@ -319,77 +321,99 @@ __device__ __forceinline__ void drift_one(const PartArgs& __restrict__ p,
     if (F32 && bend > bbeg)
 #pragma unroll
       for (int c = 0; c < 3; ++c) split_df(r1[c], r1h[c], r1l[c]);
-    for (int b = bbeg; b < bend; ++b) {
-      const long long j = d.nbr_j[b];
-      const C k = kr[2 * b], r0 = kr[2 * b + 1];
-      C ec[3];
-      C dist, D;
-      if constexpr (F32) {
-        // The bond vector e = r_j - r_i and |e|^2 - r0^2 in double-float
-        // arithmetic on the FP32 pipe: e as eh + el (TwoSum of the highs
-        // plus the difference of the lows; the minimum image subtracts n
-        // from eh exactly), |e|^2 as the exact products eh^2 (FMA residue)
-        // plus 2 eh el, summed with TwoSum against r0^2 = hi + lo.  The
-        // result matches the FP64 difference of squares to about 2^-46 |e|^2.
-        float eh[3], el[3], P[3], PE[3];
+    // two bonds at a time: their indices, constants and partner positions
+    // are loaded together (a marker's bonds are one dependent chain
+    // otherwise), the forces are added in bond order
+    for (int b0 = bbeg; b0 < bend; b0 += BONDS_AT_ONCE) {
+      long long jn[BONDS_AT_ONCE];
+      C kn[BONDS_AT_ONCE], r0n[BONDS_AT_ONCE];
+      double r0sq[BONDS_AT_ONCE], rjn[BONDS_AT_ONCE][3];
 #pragma unroll
-        for (int c = 0; c < 3; ++c) {
-          double rj = d.pos_in[c * M + j];
-          if (!d.at_force_point) rj += dt_pre01 * d.vel_in[c * M + j];
-          float jh, jl, err;
-          split_df(rj, jh, jl);
-          float sh = two_sum(jh, -r1h[c], err);
-          float t = err + (jl - r1l[c]);
-          float h = sh + t;                      // renormalised pair h + l
-          float l = t - (h - sh);
-          if (per[c]) {
-            const float half = 0.5f * (float)n3[c];
-            int shift = 0;
-            if (h > half || (h == half && l > 0.0f)) shift = -1;
-            else if (h < -half || (h == -half && l < 0.0f)) shift = 1;
-            if (shift != 0) {
-              const float hs = h + (float)(shift * n3[c]);   // exact (Sterbenz)
-              h = hs + l;
-              l = l - (h - hs);
-            }
-          }
-          eh[c] = h;
-          el[c] = l;
-          ec[c] = h;
-          P[c] = h * h;
-          PE[c] = fmaf(h, h, -P[c]) + 2.0f * h * l;
-        }
-        float e1, e2, e3, r0h, r0l;
-        const float S1 = two_sum(P[0], P[1], e1);
-        const float S2 = two_sum(S1, P[2], e2);
-        split_df(d.nbr_r0sq[b], r0h, r0l);
-        const float S3 = two_sum(S2, -r0h, e3);
-        D = S3 + (((e1 + e2) + e3) + ((PE[0] + PE[1]) + PE[2]) - r0l);
-        dist = sqrtf(S2);
-      } else {
-        double dist2 = 0.0;
-#pragma unroll
-        for (int c = 0; c < 3; ++c) {
-          double rj;
-          if (d.at_force_point) {
-            rj = d.pos_in[c * M + j];
-          } else {
-            const double vj = d.vel_in[c * M + j];
-            rj = (d.pos_in[c * M + j] + d.dt_pre0 * vj) + d.dt_pre * vj;
-          }
-          const double e = min_image(rj - r1[c], n3[c], per[c]);
-          ec[c] = (C)e;
-          dist2 += e * e;
-        }
-        // the difference of squares in FP64: bonds sit near their rest
-        // length, where |d| - r0 formed directly would lose most digits
-        dist = sqrt((C)dist2);
-        D = (C)(dist2 - d.nbr_r0sq[b]);
+      for (int q = 0; q < BONDS_AT_ONCE; ++q) {
+        const int b = b0 + q < bend ? b0 + q : b0;       // past the end: the first one again
+        jn[q] = d.nbr_j[b];
+        kn[q] = kr[2 * b];
+        r0n[q] = kr[2 * b + 1];
+        r0sq[q] = d.nbr_r0sq[b];
       }
-      // stretch |d| - r0 = (|d|^2 - r0^2) / (|d| + r0)
-      const C stretch = D / (dist + r0);
-      const C mag = k * stretch / dist;
-      for (int c = 0; c < 3; ++c) F[c] += ec[c] * mag;
+#pragma unroll
+      for (int q = 0; q < BONDS_AT_ONCE; ++q)
+#pragma unroll
+        for (int c = 0; c < 3; ++c) rjn[q][c] = d.pos_in[c * M + jn[q]];
+      if (!d.at_force_point) {
+#pragma unroll
+        for (int q = 0; q < BONDS_AT_ONCE; ++q)
+#pragma unroll
+          for (int c = 0; c < 3; ++c) {
+            const double vj = d.vel_in[c * M + jn[q]];
+            rjn[q][c] = F32 ? rjn[q][c] + dt_pre01 * vj : (rjn[q][c] + d.dt_pre0 * vj) + d.dt_pre * vj;
+          }
+      }
+#pragma unroll
+      for (int q = 0; q < BONDS_AT_ONCE; ++q) {
+        if (b0 + q >= bend) break;
+        const C k = kn[q], r0 = r0n[q];
+        C ec[3];
+        C dist, D;
+        if constexpr (F32) {
+          // The bond vector e = r_j - r_i and |e|^2 - r0^2 in double-float
+          // arithmetic on the FP32 pipe: e as eh + el (TwoSum of the highs
+          // plus the difference of the lows; the minimum image subtracts n
+          // from eh exactly), |e|^2 as the exact products eh^2 (FMA residue)
+          // plus 2 eh el, summed with TwoSum against r0^2 = hi + lo.  The
+          // result matches the FP64 difference of squares to about 2^-46 |e|^2.
+          float eh[3], el[3], P[3], PE[3];
+#pragma unroll
+          for (int c = 0; c < 3; ++c) {
+            const double rj = rjn[q][c];
+            float jh, jl, err;
+            split_df(rj, jh, jl);
+            float sh = two_sum(jh, -r1h[c], err);
+            float t = err + (jl - r1l[c]);
+            float h = sh + t;                      // renormalised pair h + l
+            float l = t - (h - sh);
+            if (per[c]) {
+              const float half = 0.5f * (float)n3[c];
+              int shift = 0;
+              if (h > half || (h == half && l > 0.0f)) shift = -1;
+              else if (h < -half || (h == -half && l < 0.0f)) shift = 1;
+              if (shift != 0) {
+                const float hs = h + (float)(shift * n3[c]);   // exact (Sterbenz)
+                h = hs + l;
+                l = l - (h - hs);
+              }
+            }
+            eh[c] = h;
+            el[c] = l;
+            ec[c] = h;
+            P[c] = h * h;
+            PE[c] = fmaf(h, h, -P[c]) + 2.0f * h * l;
+          }
+          float e1, e2, e3, r0h, r0l;
+          const float S1 = two_sum(P[0], P[1], e1);
+          const float S2 = two_sum(S1, P[2], e2);
+          split_df(r0sq[q], r0h, r0l);
+          const float S3 = two_sum(S2, -r0h, e3);
+          D = S3 + (((e1 + e2) + e3) + ((PE[0] + PE[1]) + PE[2]) - r0l);
+          dist = sqrtf(S2);
+        } else {
+          double dist2 = 0.0;
+#pragma unroll
+          for (int c = 0; c < 3; ++c) {
+            const double e = min_image(rjn[q][c] - r1[c], n3[c], per[c]);
+            ec[c] = (C)e;
+            dist2 += e * e;
+          }
+          // the difference of squares in FP64: bonds sit near their rest
+          // length, where |d| - r0 formed directly would lose most digits
+          dist = sqrt((C)dist2);
+          D = (C)(dist2 - r0sq[q]);
+        }
+        // stretch |d| - r0 = (|d|^2 - r0^2) / (|d| + r0)
+        const C stretch = D / (dist + r0);
+        const C mag = k * stretch / dist;
+        for (int c = 0; c < 3; ++c) F[c] += ec[c] * mag;
+      }
     }
     const int body = d.rigid.nbodies > 0 ? d.rigid.body_of[i] : -1;
     if (body >= 0) {
@@ -1024,12 +1048,11 @@ __device__ inline void cache_store(double* p, const double (&j)[3], double inv) 
   reinterpret_cast<double2*>(p)[1] = make_double2(j[2], inv);
 }
 
-// velocity contribution of one stencil node of weight wt from its j and
-// 1 / rho, added to own: (((j + c1 F1) + cg g) + c2 F2) / rho (F1, F2 where
-// their tile flags are set)
+// fluid velocity at one stencil node from its j and 1 / rho:
+// (((j + c1 F1) + cg g) + c2 F2) / rho (F1, F2 where their tile flags are set)
 template <typename C>
-__device__ __forceinline__ void node_add(const GatherArgs& a, long long cell, int tile, C wt,
-                                         C (&j)[3], C inv, const C (&cgg)[3], C (&own)[3]) {
+__device__ __forceinline__ void node_velocity(const GatherArgs& a, long long cell, int tile, C (&j)[3],
+                                              C inv, const C (&cgg)[3], C (&nv)[3]) {
   // each force 4-vector is loaded together with its tile's flag (it lies
   // inside the field either way) and used only where the flag is set, so
   // the two loads are not one after the other
@@ -1054,33 +1077,60 @@ __device__ __forceinline__ void node_add(const GatherArgs& a, long long cell, in
     const C c2 = rv<C>(a.c2);
     j[0] += c2 * f2x; j[1] += c2 * f2y; j[2] += c2 * f2z;
   }
-  own[0] += wt * (j[0] * inv); own[1] += wt * (j[1] * inv); own[2] += wt * (j[2] * inv);
+  nv[0] = j[0] * inv; nv[1] = j[1] * inv; nv[2] = j[2] * inv;
+}
+// the same times the node's weight wt, added to own
+template <typename C>
+__device__ __forceinline__ void node_add(const GatherArgs& a, long long cell, int tile, C wt,
+                                         C (&j)[3], C inv, const C (&cgg)[3], C (&own)[3]) {
+  C nv[3];
+  node_velocity<C>(a, cell, tile, j, inv, cgg, nv);
+  own[0] += wt * nv[0]; own[1] += wt * nv[1]; own[2] += wt * nv[2];
 }
 
 // fluid velocity at one stencil node (x, y, z) of weight wt, added to own,
-// with j and 1 / rho taken from the node cache where it is valid, else from
-// the node-moment field where its tile is ready, else pulled from the
-// populations
+// with j and 1 / rho taken from the node-moment field where its tile is
+// ready, else pulled from the populations
 template <typename S, bool WALLS>
 __device__ __forceinline__ void gather_node(const GatherArgs& a, const Geom& g, int x, int y, int z,
-                                            typename Store<S>::C wt, bool reuse,
-                                            typename Store<S>::C* slot,
+                                            typename Store<S>::C wt,
                                             const typename Store<S>::C (&cgg)[3],
                                             typename Store<S>::C (&own)[3]) {
   using C = typename Store<S>::C;
   C j[3], inv;
   const long long cell = z * g.plane + (long long)y * g.pitch + x;
   const int tile = tile_of(g, x, y, z);
-  if (reuse) {
-    cache_load(slot, j, inv);
-  } else {
-    if (a.mom != nullptr && a.mready[tile])
-      cache_load(static_cast<const C*>(a.mom) + 4 * cell, j, inv);
-    else
-      node_base<S, WALLS>(a, g, x, y, z, j, inv);
-    if (a.cache != 0) cache_store(slot, j, inv);
-  }
+  if (a.mom != nullptr && a.mready[tile])
+    cache_load(static_cast<const C*>(a.mom) + 4 * cell, j, inv);
+  else
+    node_base<S, WALLS>(a, g, x, y, z, j, inv);
   node_add<C>(a, cell, tile, wt, j, inv, cgg, own);
+}
+
+// the next step's binning from a marker's end-of-step position: its tile key
+// and index, and the flag that requests a re-sort (FP32 compute: the float
+// splits of the coordinates, as the key-writing drift)
+template <typename C>
+__device__ __forceinline__ void next_bin(const GatherArgs& a, const Geom& g, long long i,
+                                         const double (&rn)[3]) {
+  constexpr bool F32 = sizeof(C) == 4;
+  a.key_out[i] = F32 ? key_of_f(g, rn[0], rn[1], rn[2]) : key_of(g, rn[0], rn[1], rn[2]);
+  a.idx_out[i] = (uint32_t)i;
+  if (a.home && !(F32 ? near_home_f(g, a.home[i], rn) : near_home(g, a.home[i], rn))) *a.need_next = 1;
+}
+
+// the stencil record of slot k and its packed base
+template <int ST, typename C>
+__device__ __forceinline__ void write_record(const GatherArgs& a, long long k, const int (&b)[3],
+                                             const C (&w)[3][4], const C (&F)[3]) {
+  StencilRecT<C> r;
+  r.bx = b[0]; r.by = b[1]; r.bz = b[2]; r.kind = ST;
+#pragma unroll
+  for (int q = 0; q < 4; ++q) { r.wx[q] = w[0][q]; r.wy[q] = w[1][q]; r.wz[q] = w[2][q]; }
+  r.F[0] = F[0]; r.F[1] = F[1]; r.F[2] = F[2];
+  r.pad = C(0);
+  static_cast<StencilRecT<C>*>(a.rec)[k] = r;
+  a.reach[k] = pack_base(b[0], b[1], b[2]);
 }
 
 // v[q] by selects (the array stays in registers)
@@ -1137,17 +1187,207 @@ __device__ __forceinline__ bool gather_field(const GatherArgs& a, const Geom& g,
   return ok;
 }
 
-// Variants (VAR): GV_FULL keeps registers for the population loads of two
-// nodes at a time; GV_LIGHT is launched for sub-steps that read the node
-// cache or the node-moment field (fewer registers, more markers in flight);
-// GV_QUAD (4- and 3-point stencils, no node cache, no fused drift; by
-// default only for fewer markers than the one-lane variants keep resident
-// at once) gives each marker four lanes, lane q taking the stencil rows ky = q (mod 4) of
-// every plane, and sums their parts with a fixed butterfly: four times the
-// loads in flight for the same markers.  Lane 0 of a group does the
-// marker's update and writes its record; the tile claims are shared out by
-// plane.
-constexpr int GV_FULL = 0, GV_LIGHT = 1, GV_QUAD = 2;
+// Variants (VAR) of the interpolation:
+//   GV_FULL    one lane per marker, no node cache: pulls the populations of
+//              two nodes at a time (or reads the node-moment field);
+//   GV_LIGHT   the same for launches that read the node-moment field (fewer
+//              registers, more markers in flight);
+//   GV_QUAD    (4- and 3-point stencils, no node cache, no fused drift; by
+//              default only for fewer markers than the one-lane variants
+//              keep resident at once) four lanes per marker, lane q taking
+//              the stencil rows ky = q (mod 4) of every plane, their parts
+//              summed with a fixed butterfly: four times the loads in flight
+//              for the same markers.  Lane 0 of a group does the marker's
+//              update and writes its record; the tile claims are shared out
+//              by plane;
+//   GV_CACHED  one lane per marker with the node cache: markers whose cache
+//              entry does not hold are refilled by the whole warp first
+//              (refill_cache), then every lane reads its nodes from the
+//              cache with all loads in flight;
+//   GV_OCT     (trilinear) eight lanes per marker, one per node
+//              (gather_oct_body).
+constexpr int GV_FULL = 0, GV_LIGHT = 1, GV_QUAD = 2, GV_CACHED = 3, GV_OCT = 4;
+
+// Coupling force F^h of N components from the slip dv = v - u(X), the
+// intrinsic force Fi and the random force zeta (compute type)
+template <typename C, int N>
+__device__ __forceinline__ void couple_force(const GatherArgs& __restrict__ a, C cim, const C (&dv)[N],
+                                             const C (&Fi)[N], const C (&zeta)[N], C (&Fh)[N]) {
+  const C cs = rv<C>(a.s), crho = rv<C>(a.rho0);
+  if (a.kind == 4) {                        // modified EBF, Eq. [modified-ebf]
+    // r = 1/(1 + m/rho0) = rho0 im/(rho0 im + 1); 1/(s(1/m + 1/rho0))
+    const C r = crho * cim / (crho * cim + C(1));
+    const C inv = C(1) / (cs * (cim + C(1) / crho));
+#pragma unroll
+    for (int c = 0; c < N; ++c) Fh[c] = -dv[c] * inv - r * Fi[c];
+  } else {
+    const C gam = a.kind == 3 ? crho : rv<C>(a.gamma);   // EBF: rho a^3 / h
+    if (a.order == 1) {
+#pragma unroll
+      for (int c = 0; c < N; ++c) Fh[c] = -gam * dv[c];
+      if (a.noise)
+#pragma unroll
+        for (int c = 0; c < N; ++c) Fh[c] += zeta[c];
+    } else {                                // Crank-Nicolson, Eq. [modified-force]
+      const C al = gam * cs * cim, be = gam * cs / crho;
+      const C D = C(1) + C(0.5) * al + C(0.5) * be;
+      if (a.noise) {
+#pragma unroll
+        for (int c = 0; c < N; ++c) Fh[c] = -((gam * dv[c] + C(0.5) * al * Fi[c]) - zeta[c]) / D;
+      } else {
+#pragma unroll
+        for (int c = 0; c < N; ++c) Fh[c] = -(gam * dv[c] + C(0.5) * al * Fi[c]) / D;
+      }
+    }
+  }
+}
+
+// The tile of stencil node q of an axis, or -1 if it carries no weight, lies
+// outside the box or repeats an earlier node's tile
+template <int SN, typename C>
+__device__ __forceinline__ void axis_tiles(int b, const C (&w)[4], int n, bool periodic, int (&tq)[SN]) {
+#pragma unroll
+  for (int q = 0; q < SN; ++q) {
+    int t = -1;
+    if (w[q] != C(0)) {
+      int node = b + q;
+      if (periodic) node = wrap_int(node, n);
+      if (node >= 0 && node < n) t = node >> TILE_SHIFT;
+    }
+#pragma unroll
+    for (int e = 0; e < q; ++e) if (tq[e] == t) t = -1;
+    tq[q] = t;
+  }
+}
+
+// the bins are valid while every stencil node lies within three cells of the
+// home tile (the reach of the spreading's neighbour search)
+template <int SN>
+__device__ __forceinline__ bool bins_hold(const Geom& g, int home, const int (&b)[3]) {
+  const unsigned t = (unsigned)home, r = t / (unsigned)g.ntx, tz = r / (unsigned)g.nty;
+  const int tt[3] = {(int)(t - r * g.ntx), (int)(r - tz * g.nty), (int)tz};
+  const int n3[3] = {g.nx, g.ny, g.nz};
+  bool ok = true;
+#pragma unroll
+  for (int c = 0; c < 3; ++c) {
+    const int lo = tt[c] * TILE, hi = min(lo + TILE, n3[c]) - 1;
+    ok = ok && stencil_near_home<SN>(b[c], lo, hi, n3[c], c < 2 || !g.walls);
+  }
+  return ok;
+}
+
+// Cached variant: the whole warp fills the cache entries of its lanes'
+// markers with `want` set.  The lanes take the nodes of those markers side by
+// side (trilinear: eight nodes of four markers per round; three-point: one
+// marker, four-point: one marker in two rounds), so the 19 loads of a node
+// are in flight for 32 nodes at once and neighbouring nodes share sectors.
+// When every lane pulled its own marker's nodes one after the other, one
+// lane whose base had changed held its warp, and with it the kernel, for as
+// long as filling everything: 12 500 markers (98 blocks) 28 us per sub-step,
+// 18.5 us with the shared refill, of which the kernel's chain of about 2900
+// instructions per warp is what is left.
+template <typename S, bool WALLS, int SN>
+__device__ __forceinline__ void refill_cache(const GatherArgs& __restrict__ a, const Geom& g,
+                                             long long M, long long gid, const int (&b)[3], bool want) {
+  using C = typename Store<S>::C;
+  constexpr unsigned full = 0xffffffffu;
+  constexpr int NN = SN * SN * SN;
+  constexpr int PER = NN <= 32 ? 32 / NN : 1;          // markers per round
+  const int lane = threadIdx.x & 31;
+  C* nc = static_cast<C*>(a.ncache);
+  unsigned todo = __ballot_sync(full, want);
+  const int r = NN <= 32 ? lane / NN : 0;              // the lane's marker of the round
+  while (todo != 0u) {
+    unsigned t = todo;
+#pragma unroll
+    for (int e = 0; e < PER; ++e) {
+      if (e < r) t &= t - 1u;                          // drop the markers of other lanes
+      todo &= todo - 1u;
+    }
+    const bool have = t != 0u && r < PER;
+    const int src = have ? __ffs(t) - 1 : 0;
+    const int bx = __shfl_sync(full, b[0], src), by = __shfl_sync(full, b[1], src),
+              bz = __shfl_sync(full, b[2], src);
+    const long long kk = gid - lane + src;             // slots follow the lanes
+    if (have) {
+      for (int node = lane - r * NN; node < NN; node += 32) {
+        const int qx = node % SN, qy = (node / SN) % SN, qz = node / (SN * SN);
+        const int x = wrap_int(bx + qx, g.nx), y = wrap_int(by + qy, g.ny);
+        int z = bz + qz;
+        if (!WALLS) z = wrap_int(z, g.nz);
+        if (WALLS && (z < 0 || z >= g.nz)) continue;
+        C j[3], inv;
+        node_base<S, WALLS>(a, g, x, y, z, j, inv);
+        cache_store(nc + (node * M + kk) * 4, j, inv);
+      }
+    }
+  }
+  __syncwarp();                                        // the entries are read by their owners
+}
+
+// Fluid velocity from the cached trilinear nodes, F1 and F2 present or not
+// at compile time: the node, force and flag loads of a plane of nodes are
+// issued together, then added in node order.
+template <typename C, bool HAS1, bool HAS2>
+__device__ __forceinline__ void cached_nodes(const GatherArgs& __restrict__ a, const Geom& g, long long M,
+                                             long long k, const int (&xs)[2], const int (&ys)[2],
+                                             const int (&zs)[2], const C (&w)[3][4], const C (&cgg)[3],
+                                             C (&own)[3]) {
+  const C* nc = static_cast<const C*>(a.ncache) + 4 * k;
+  const C* F1 = static_cast<const C*>(a.F1);
+  const C* F2 = static_cast<const C*>(a.F2);
+  const C c1 = rv<C>(a.c1), c2 = rv<C>(a.c2);
+#pragma unroll
+  for (int kz = 0; kz < 2; ++kz) {
+    if (zs[kz] < 0) continue;                          // beyond a wall
+    C j[4][3], inv[4], f1[4][3], f2[4][3];
+    bool on1[4], on2[4];
+#pragma unroll
+    for (int q = 0; q < 4; ++q) {
+      const int y = ys[q >> 1], x = xs[q & 1];
+      cache_load(nc + (4 * kz + q) * M * 4, j[q], inv[q]);
+      const long long cell = zs[kz] * g.plane + (long long)y * g.pitch + x;
+      const int tile = tile_of(g, x, y, zs[kz]);
+      if (HAS1) {
+        on1[q] = a.flag1[tile] != 0;
+        load_force(F1, cell, f1[q][0], f1[q][1], f1[q][2]);
+      }
+      if (HAS2) {
+        on2[q] = a.flag2[tile] != 0;
+        load_force(F2, cell, f2[q][0], f2[q][1], f2[q][2]);
+      }
+    }
+#pragma unroll
+    for (int q = 0; q < 4; ++q) {
+      const C wt = w[0][q & 1] * (w[1][q >> 1] * w[2][kz]);
+#pragma unroll
+      for (int c = 0; c < 3; ++c) {
+        C v = j[q][c];
+        if (HAS1) v = on1[q] ? v + c1 * f1[q][c] : v;
+        v += cgg[c];
+        if (HAS2) v = on2[q] ? v + c2 * f2[q][c] : v;
+        own[c] += wt * (v * inv[q]);
+      }
+    }
+  }
+}
+
+// List slots for the tiles claimed by the warp's lanes (nclaim each), one
+// atomic per warp: the lane's first slot.  `am`: the lanes taking part (the
+// first nact of the warp).
+__device__ __forceinline__ int claim_slots(int* nlive, int nclaim, unsigned am, int nact) {
+  const int lane = threadIdx.x & 31;
+  int incl = nclaim;
+#pragma unroll
+  for (int off = 1; off < 32; off <<= 1) {
+    const int u = __shfl_up_sync(am, incl, off);
+    if (lane >= off) incl += u;
+  }
+  const int total = __shfl_sync(am, incl, nact - 1);
+  int base = 0;
+  if (lane == nact - 1 && total > 0) base = atomicAdd(nlive, total);
+  return __shfl_sync(am, base, nact - 1) + incl - nclaim;
+}
 
 // the body of the gather for thread gid of one box's launch (whole warps of
 // one box: gid - lane is a multiple of 32)
@@ -1157,15 +1397,26 @@ __device__ __forceinline__ void gather_body(const PartArgs& __restrict__ p,
   using C = typename Store<S>::C;
   constexpr int SN = nodes_1d<ST>();
   constexpr int GL = VAR == GV_QUAD ? 4 : 1;       // lanes per marker
+  constexpr bool CACHED = VAR == GV_CACHED;
   const Geom& g = p.g;
   const long long M = p.M;
   const int lane = threadIdx.x & 31;
-  const long long k = gid / GL;
+  // the lanes still running: whole groups, the first nact of the warp; with
+  // the cache every lane stays (the refill is the whole warp's work), the
+  // ones past the last marker on the last marker and without writing
+  if (!CACHED && gid / GL >= M) return;
+  const bool valid = gid / GL < M;
+  const long long k = valid ? gid / GL : M - 1;
   const int sub = (int)(gid % GL);
-  if (k >= M) return;                  // whole groups leave together
   const long long i = a.perm ? (long long)a.perm[k] : k;
   const int n3[3] = {g.nx, g.ny, g.nz};
   const bool per[3] = {true, true, !g.walls};
+  int4 cb = make_int4(0, 0, 0, 0);
+  bool try_reuse = false;
+  if (CACHED && a.cache == 2) {
+    cb = a.ncache_b[k];
+    try_reuse = a.invalidate == nullptr || *a.invalidate == 0;
+  }
 
   // the particle's own data (independent of the gather); with a fused
   // drift this thread first does its marker's drift sub-step
@@ -1174,10 +1425,11 @@ __device__ __forceinline__ void gather_body(const PartArgs& __restrict__ p,
   C Fi[3] = {C(0), C(0), C(0)};
   double X[3];
   const bool at_aux = a.mode == GM_IBM_HALF || a.mode == GM_IBM_FINAL;
+  const int home = a.keys ? (int)a.keys[k] : 0;
   if (GL == 1 && a.fused) {
     C F[3];
-    drift_one<C>(p, a.drift, i, X, v, F);
     im = a.inv_mass[i];
+    drift_one<C>(p, a.drift, i, X, v, F);
     if (a.include_int)
 #pragma unroll
       for (int c = 0; c < 3; ++c) Fi[c] = F[c];
@@ -1198,8 +1450,7 @@ __device__ __forceinline__ void gather_body(const PartArgs& __restrict__ p,
 #pragma unroll
     for (int c = 0; c < 3; ++c) X[c] = P[c * M + i];
   }
-  const int home = a.keys ? (int)a.keys[k] : 0;
-  if (k == 0 && sub == 0 && a.clear_next) {      // the next step's flags (read by none now)
+  if (valid && k == 0 && sub == 0 && a.clear_next) {      // the next step's flags (read by none now)
     a.clear_next[0] = 0;
     a.clear_next[1] = 0;
   }
@@ -1228,57 +1479,81 @@ __device__ __forceinline__ void gather_body(const PartArgs& __restrict__ p,
       zs[q] = WALLS ? ((zz < 0 || zz >= g.nz) ? -1 : zz) : wrap_int(zz, g.nz);
     }
     const C cgg[3] = {rv<C>(a.cgg[0]), rv<C>(a.cgg[1]), rv<C>(a.cgg[2])};
-    C* nc = static_cast<C*>(a.ncache);
-    bool reuse = false;
-    if (GL == 1 && a.cache == 2 && (a.invalidate == nullptr || *a.invalidate == 0)) {
-      const int4 cb = a.ncache_b[k];
-      reuse = cb.x == b[0] && cb.y == b[1] && cb.z == b[2];
-    }
-    if (GL == 1 && a.cache != 0 && !reuse) a.ncache_b[k] = make_int4(b[0], b[1], b[2], 0);
-    bool done = false;
-    if (a.mom != nullptr && a.cache == 0) {
-      done = gather_field<S, WALLS, SN, GL>(a, g, xs, ys, zs, w, sub, cgg, own);
-      if (!done) own[0] = own[1] = own[2] = C(0);
-    }
     // node (kx, ky, kz) of slot k sits at nc[((kz SN + ky) SN + kx) M + k] (x 4)
-    if (done) {
-    } else if (SN == 2) {
+    if constexpr (CACHED) {
+      const bool reuse = try_reuse && cb.x == b[0] && cb.y == b[1] && cb.z == b[2];
+      const bool want = valid && !reuse;
+      if (want) a.ncache_b[k] = make_int4(b[0], b[1], b[2], 0);
+      refill_cache<S, WALLS, SN>(a, g, M, gid, b, want);
+      if constexpr (SN == 2) {
+        if (a.F1 != nullptr) {
+          if (a.F2 != nullptr) cached_nodes<C, true, true>(a, g, M, k, xs, ys, zs, w, cgg, own);
+          else cached_nodes<C, true, false>(a, g, M, k, xs, ys, zs, w, cgg, own);
+        } else {
+          if (a.F2 != nullptr) cached_nodes<C, false, true>(a, g, M, k, xs, ys, zs, w, cgg, own);
+          else cached_nodes<C, false, false>(a, g, M, k, xs, ys, zs, w, cgg, own);
+        }
+      } else {
+        const C* nc = static_cast<const C*>(a.ncache);
+#pragma unroll 1
+        for (int kz = 0; kz < SN; ++kz) {
+          const int z = pick(zs, kz);
+          if (WALLS && z < 0) continue;
+          const C wz = pick(w[2], kz);
+#pragma unroll 1
+          for (int ky = 0; ky < SN; ++ky) {
+            const int y = pick(ys, ky);
+            const C wyz = pick(w[1], ky) * wz;
 #pragma unroll
-      for (int kz = 0; kz < SN; ++kz)
-#pragma unroll
-        for (int ky = 0; ky < SN; ++ky)
-#pragma unroll
-          for (int kx = 0; kx < SN; ++kx) {
-            if (WALLS && zs[kz] < 0) continue;
-            const C wt = w[0][kx] * (w[1][ky] * w[2][kz]);
-            C* slot = nc + (((kz * SN + ky) * SN + kx) * M + k) * 4;
-            gather_node<S, WALLS>(a, g, xs[kx], ys[ky], zs[kz], wt, reuse, slot, cgg, own);
+            for (int kx = 0; kx < SN; ++kx) {
+              C j[3], inv;
+              cache_load(nc + (((kz * SN + ky) * SN + kx) * M + k) * 4, j, inv);
+              const long long cell = z * g.plane + (long long)y * g.pitch + xs[kx];
+              node_add<C>(a, cell, tile_of(g, xs[kx], y, z), w[0][kx] * wyz, j, inv, cgg, own);
+            }
           }
+        }
+      }
     } else {
-      // the loops are not unrolled: the per-axis nodes and weights are
-      // picked by selects, which keeps them in registers
+      bool done = false;
+      if (a.mom != nullptr) {
+        done = gather_field<S, WALLS, SN, GL>(a, g, xs, ys, zs, w, sub, cgg, own);
+        if (!done) own[0] = own[1] = own[2] = C(0);
+      }
+      if (done) {
+      } else if (SN == 2) {
+#pragma unroll
+        for (int kz = 0; kz < SN; ++kz)
+#pragma unroll
+          for (int ky = 0; ky < SN; ++ky)
+#pragma unroll
+            for (int kx = 0; kx < SN; ++kx) {
+              if (WALLS && zs[kz] < 0) continue;
+              const C wt = w[0][kx] * (w[1][ky] * w[2][kz]);
+              gather_node<S, WALLS>(a, g, xs[kx], ys[ky], zs[kz], wt, cgg, own);
+            }
+      } else {
+        // the loops are not unrolled: the per-axis nodes and weights are
+        // picked by selects, which keeps them in registers
 #pragma unroll 1
-      for (int kz = 0; kz < SN; ++kz) {
-        const int z = pick(zs, kz);
-        if (WALLS && z < 0) continue;
-        const C wz = pick(w[2], kz);
+        for (int kz = 0; kz < SN; ++kz) {
+          const int z = pick(zs, kz);
+          if (WALLS && z < 0) continue;
+          const C wz = pick(w[2], kz);
 #pragma unroll 1
-        for (int ky = sub; ky < SN; ky += GL) {
-          const int y = pick(ys, ky);
-          const C wyz = pick(w[1], ky) * wz;
+          for (int ky = sub; ky < SN; ky += GL) {
+            const int y = pick(ys, ky);
+            const C wyz = pick(w[1], ky) * wz;
 #pragma unroll 2
-          for (int kx = 0; kx < SN; ++kx) {
-            C* slot = nc + (((kz * SN + ky) * SN + kx) * M + k) * 4;
-            gather_node<S, WALLS>(a, g, pick(xs, kx), y, z, pick(w[0], kx) * wyz, reuse, slot, cgg,
-                                  own);
+            for (int kx = 0; kx < SN; ++kx)
+              gather_node<S, WALLS>(a, g, pick(xs, kx), y, z, pick(w[0], kx) * wyz, cgg, own);
           }
         }
       }
     }
   }
-  // the warp's lanes still running are its first nact (whole groups)
   const long long wbase = gid - lane;
-  const int nact = M * GL - wbase >= 32 ? 32 : (int)(M * GL - wbase);
+  const int nact = CACHED || M * GL - wbase >= 32 ? 32 : (int)(M * GL - wbase);
   const unsigned am = nact == 32 ? 0xffffffffu : ((1u << nact) - 1u);
   if (GL > 1) {
 #pragma unroll
@@ -1291,43 +1566,21 @@ __device__ __forceinline__ void gather_body(const PartArgs& __restrict__ p,
   // stencil record and tile claims
   const double s = a.s.d;
   C Frec[3] = {C(0), C(0), C(0)};
-  switch (sub == 0 ? a.mode : -1) {
+  switch (sub == 0 && valid ? a.mode : -1) {
     case GM_COUPLE: {
       // slip v - u(X) in the compute type (FP64 work being scarce): with
       // FP32 the rounding of v adds at most 2^-24 |v| to it
-      C dv[3];
+      C dv[3], zeta[3] = {C(0), C(0), C(0)}, Fh[3];
       for (int c = 0; c < 3; ++c) dv[c] = (C)v[c] - own[c];
-      C Fh[3];
-      const C cs = rv<C>(a.s), cim = C(im), crho = rv<C>(a.rho0);
-      if (a.kind == 4) {                      // modified EBF, Eq. [modified-ebf]
-        // r = 1/(1 + m/rho0) = rho0 im/(rho0 im + 1); 1/(s(1/m + 1/rho0))
-        const C r = crho * cim / (crho * cim + C(1));
-        const C inv = C(1) / (cs * (cim + C(1) / crho));
-        for (int c = 0; c < 3; ++c) Fh[c] = -dv[c] * inv - r * Fi[c];
-      } else {
-        const C gam = a.kind == 3 ? crho : rv<C>(a.gamma);   // EBF: rho a^3 / h
-        // the random force zeta of this (sub-)step (thermal boxes)
-        C zeta[3] = {C(0), C(0), C(0)};
-        if (a.noise) {
-          C r[4];
-          philox_gauss4<C>((uint32_t)i, (uint32_t)(*a.tstep), 8u + (uint32_t)a.substep, 0u,
-                           a.tkey0, a.tkey1, r);
-          const C za = rv<C>(a.zeta_amp);
-          for (int c = 0; c < 3; ++c) zeta[c] = za * r[c];
-        }
-        if (a.order == 1) {
-          for (int c = 0; c < 3; ++c) Fh[c] = -gam * dv[c];
-          if (a.noise)
-            for (int c = 0; c < 3; ++c) Fh[c] += zeta[c];
-        } else {                              // Crank-Nicolson, Eq. [modified-force]
-          const C al = gam * cs * cim, be = gam * cs / crho;
-          const C D = C(1) + C(0.5) * al + C(0.5) * be;
-          if (a.noise)
-            for (int c = 0; c < 3; ++c) Fh[c] = -((gam * dv[c] + C(0.5) * al * Fi[c]) - zeta[c]) / D;
-          else
-            for (int c = 0; c < 3; ++c) Fh[c] = -(gam * dv[c] + C(0.5) * al * Fi[c]) / D;
-        }
+      // the random force zeta of this (sub-)step (thermal boxes)
+      if (a.noise) {
+        C r[4];
+        philox_gauss4<C>((uint32_t)i, (uint32_t)(*a.tstep), 8u + (uint32_t)a.substep, 0u,
+                         a.tkey0, a.tkey1, r);
+        const C za = rv<C>(a.zeta_amp);
+        for (int c = 0; c < 3; ++c) zeta[c] = za * r[c];
       }
+      couple_force<C, 3>(a, C(im), dv, Fi, zeta, Fh);
       const double kick = s * im;
       double vn[3];
       for (int c = 0; c < 3; ++c) {
@@ -1348,11 +1601,7 @@ __device__ __forceinline__ void gather_body(const PartArgs& __restrict__ p,
                             n3[c], per[c]);
           a.pos_next[c * M + i] = rn[c];
         }
-        if (a.key_out) {            // the next step's binning, from these positions
-          a.key_out[i] = key_of(g, rn[0], rn[1], rn[2]);
-          a.idx_out[i] = (uint32_t)i;
-          if (a.home && !near_home(g, a.home[i], rn)) *a.need_next = 1;
-        }
+        if (a.key_out) next_bin<C>(a, g, i, rn);
       }
       break;
     }
@@ -1375,191 +1624,91 @@ __device__ __forceinline__ void gather_body(const PartArgs& __restrict__ p,
       break;
   }
   if (a.rec && (a.mode == GM_COUPLE || a.mode == GM_IBM_HALF || a.mode == GM_IBM1)) {
+    if (sub == 0 && valid) {
+      write_record<ST>(a, k, b, w, Frec);
+      if (a.keys && !bins_hold<SN>(g, home, b)) *a.status = 1;
+    }
     if constexpr (SN == 2) {
-      // trilinear: the 2 x 2 x 2 node combinations, unrolled
-      unsigned long long claimed = 0ull;   // bit (qz SN + qy) SN + qx
-      int nclaim = 0;
+      // trilinear: the 2 x 2 x 2 node combinations, unrolled.  The marker
+      // joins the hit list of every tile it reaches; the first to join
+      // claims the tile.  All the joins are issued before any of their
+      // counts is looked at.
       int tq[3][SN];
-      {
-        if (sub == 0) {
-          StencilRecT<C> r;
-          r.bx = b[0]; r.by = b[1]; r.bz = b[2]; r.kind = ST;
-          for (int q = 0; q < 4; ++q) { r.wx[q] = w[0][q]; r.wy[q] = w[1][q]; r.wz[q] = w[2][q]; }
-          r.F[0] = Frec[0]; r.F[1] = Frec[1]; r.F[2] = Frec[2];
-          r.pad = C(0);
-          static_cast<StencilRecT<C>*>(a.rec)[k] = r;
-          a.reach[k] = pack_base(b[0], b[1], b[2]);
+#pragma unroll
+      for (int c = 0; c < 3; ++c) axis_tiles<SN>(b[c], w[c], n3[c], per[c], tq[c]);
+      uint32_t slot[8];
+      unsigned joined = 0u;
+#pragma unroll
+      for (int q = 0; q < 8; ++q) {
+        const int tx = tq[0][q & 1], ty = tq[1][(q >> 1) & 1], tz = tq[2][q >> 2];
+        slot[q] = 1u;
+        if (valid && tx >= 0 && ty >= 0 && tz >= 0) {
+          slot[q] = atomicAdd(a.hcnt + (tz * g.nty + ty) * g.ntx + tx, 1u);
+          joined |= 1u << q;
         }
-        // claim the tiles the stencil reaches (nodes with non-zero weight); per
-        // axis tq[c][q] is the tile of node q, or -1 if it repeats an earlier
-        // node's tile or carries no weight
+      }
+      unsigned claimed = 0u;
 #pragma unroll
-        for (int c = 0; c < 3; ++c) {
-#pragma unroll
-          for (int q = 0; q < SN; ++q) {
-            int t = -1;
-            if (w[c][q] != C(0)) {
-              int node = b[c] + q;
-              if (per[c]) node = wrap_int(node, n3[c]);
-              if (node >= 0 && node < n3[c]) t = node >> TILE_SHIFT;
-            }
-#pragma unroll
-            for (int e = 0; e < q; ++e) if (tq[c][e] == t) t = -1;
-            tq[c][q] = t;
+      for (int q = 0; q < 8; ++q)
+        if (joined & (1u << q)) {
+          const int tile = (tq[2][q >> 2] * g.nty + tq[1][(q >> 1) & 1]) * g.ntx + tq[0][q & 1];
+          if (slot[q] < (uint32_t)SPREAD_HCAP)
+            a.hits[(size_t)tile * SPREAD_HCAP + slot[q]] = (uint32_t)k;
+          if (slot[q] == 0u) {
+            a.mark[tile] = 1u;
+            claimed |= 1u << q;
           }
         }
+      int base = claim_slots(a.nlive, __popc(claimed), am, nact);
 #pragma unroll
-        for (int qz = 0; qz < SN; ++qz)
-#pragma unroll
-          for (int qy = 0; qy < SN; ++qy)
-#pragma unroll
-            for (int qx = 0; qx < SN; ++qx)
-              if (qz % GL == sub && tq[2][qz] >= 0 && tq[1][qy] >= 0 && tq[0][qx] >= 0) {
-                const int tile = (tq[2][qz] * g.nty + tq[1][qy]) * g.ntx + tq[0][qx];
-                bool first;
-                if (a.hcnt != nullptr) {
-                  // the marker joins the tile's hit list; the first to join
-                  // claims the tile
-                  const uint32_t slot = atomicAdd(a.hcnt + tile, 1u);
-                  if (slot < (uint32_t)SPREAD_HCAP)
-                    a.hits[(size_t)tile * SPREAD_HCAP + slot] = (uint32_t)k;
-                  first = slot == 0u;
-                  if (first) a.mark[tile] = 1u;
-                } else {
-                  // most tiles are claimed already: an L2 read (marks only go
-                  // from 0 to 1 during the gather) spares their atomic
-                  uint32_t* m = a.mark + tile;
-                  first = __ldcg(m) == 0u && atomicExch(m, 1u) == 0u;
-                }
-                if (first) {
-                  claimed |= 1ull << ((qz * SN + qy) * SN + qx);
-                  ++nclaim;
-                }
-              }
-        if (a.keys && sub == 0) {
-          // the bins are valid while every stencil node lies within three
-          // cells of the home tile (the reach of the spreading's neighbour
-          // search)
-          const int t = home;
-          const int tt[3] = {t % g.ntx, (t / g.ntx) % g.nty, t / (g.ntx * g.nty)};
-          bool ok = true;
-          for (int c = 0; c < 3; ++c) {
-            const int lo = tt[c] * TILE, hi = min(lo + TILE, n3[c]) - 1;
-            ok = ok && stencil_near_home<SN>(b[c], lo, hi, n3[c], per[c]);
-          }
-          if (!ok) *a.status = 1;
+      for (int q = 0; q < 8; ++q)
+        if (claimed & (1u << q)) {
+          const int tx = tq[0][q & 1], ty = tq[1][(q >> 1) & 1], tz = tq[2][q >> 2];
+          a.live_tiles[base++] = make_int4((tz * g.nty + ty) * g.ntx + tx, tx, ty, tz);
         }
-    }
-      // list slots for the claimed tiles, one atomic per warp
-      int incl = nclaim;
-#pragma unroll
-      for (int off = 1; off < 32; off <<= 1) {
-        const int u = __shfl_up_sync(am, incl, off);
-        if (lane >= off) incl += u;
-    }
-      const int total = __shfl_sync(am, incl, nact - 1);
-      int base = 0;
-      if (lane == nact - 1 && total > 0) base = atomicAdd(a.nlive, total);
-      base = __shfl_sync(am, base, nact - 1) + incl - nclaim;
-#pragma unroll
-      for (int qz = 0; qz < SN; ++qz)
-#pragma unroll
-        for (int qy = 0; qy < SN; ++qy)
-#pragma unroll
-          for (int qx = 0; qx < SN; ++qx)
-            if (claimed & (1ull << ((qz * SN + qy) * SN + qx)))
-              a.live_tiles[base++] = make_int4((tq[2][qz] * g.nty + tq[1][qy]) * g.ntx + tq[0][qx],
-                                               tq[0][qx], tq[1][qy], tq[2][qz]);
     } else {
       // 4- and 3-point stencils: loops over the distinct tiles per axis
-      // instead of the SN^3 node combinations
-      // per axis the distinct tiles of the nodes with non-zero weight, in
-      // node order (at most three: a partial last tile and the periodic wrap)
+      // instead of the SN^3 node combinations: per axis the distinct tiles
+      // of the nodes with non-zero weight, in node order (at most three: a
+      // partial last tile and the periodic wrap)
       int tl[3][3], ntl[3];
       uint32_t claimed = 0u;               // bit of the tile combination cid
       int nclaim = 0;
-      {
-        if (sub == 0) {
-          StencilRecT<C> r;
-          r.bx = b[0]; r.by = b[1]; r.bz = b[2]; r.kind = ST;
-          for (int q = 0; q < 4; ++q) { r.wx[q] = w[0][q]; r.wy[q] = w[1][q]; r.wz[q] = w[2][q]; }
-          r.F[0] = Frec[0]; r.F[1] = Frec[1]; r.F[2] = Frec[2];
-          r.pad = C(0);
-          static_cast<StencilRecT<C>*>(a.rec)[k] = r;
-          a.reach[k] = pack_base(b[0], b[1], b[2]);
-        }
 #pragma unroll
-        for (int c = 0; c < 3; ++c) {
-          ntl[c] = 0;
-          tl[c][0] = tl[c][1] = tl[c][2] = -1;
+      for (int c = 0; c < 3; ++c) {
+        ntl[c] = 0;
+        tl[c][0] = tl[c][1] = tl[c][2] = -1;
 #pragma unroll
-          for (int q = 0; q < SN; ++q) {
-            if (w[c][q] == C(0)) continue;
-            int node = b[c] + q;
-            if (per[c]) node = wrap_int(node, n3[c]);
-            if (node < 0 || node >= n3[c]) continue;
-            const int t = node >> TILE_SHIFT;
-            if (t == tl[c][0] || t == tl[c][1] || t == tl[c][2]) continue;
-            if (ntl[c] == 0) tl[c][0] = t;
-            else if (ntl[c] == 1) tl[c][1] = t;
-            else tl[c][2] = t;
-            ++ntl[c];
-          }
+        for (int q = 0; q < SN; ++q) {
+          if (w[c][q] == C(0)) continue;
+          int node = b[c] + q;
+          if (per[c]) node = wrap_int(node, n3[c]);
+          if (node < 0 || node >= n3[c]) continue;
+          const int t = node >> TILE_SHIFT;
+          if (t == tl[c][0] || t == tl[c][1] || t == tl[c][2]) continue;
+          if (ntl[c] == 0) tl[c][0] = t;
+          else if (ntl[c] == 1) tl[c][1] = t;
+          else tl[c][2] = t;
+          ++ntl[c];
         }
-        // claim the tiles the stencil reaches: the combinations of the axes'
-        // tiles, shared out over the marker's lanes
-        int cid = 0;
-        for (int iz = 0; iz < ntl[2]; ++iz)
-          for (int iy = 0; iy < ntl[1]; ++iy)
-            for (int ix = 0; ix < ntl[0]; ++ix, ++cid) {
-              if (cid % GL != sub) continue;
-              const int tx = pick(tl[0], ix), ty = pick(tl[1], iy), tz = pick(tl[2], iz);
-              const int tile = (tz * g.nty + ty) * g.ntx + tx;
-              bool first;
-              if (a.hcnt != nullptr) {
-                // the marker joins the tile's hit list; the first to join
-                // claims the tile
-                const uint32_t slot = atomicAdd(a.hcnt + tile, 1u);
-                if (slot < (uint32_t)SPREAD_HCAP)
-                  a.hits[(size_t)tile * SPREAD_HCAP + slot] = (uint32_t)k;
-                first = slot == 0u;
-                if (first) a.mark[tile] = 1u;
-              } else {
-                // most tiles are claimed already: an L2 read (marks only go
-                // from 0 to 1 during the gather) spares their atomic
-                uint32_t* m = a.mark + tile;
-                first = __ldcg(m) == 0u && atomicExch(m, 1u) == 0u;
-              }
-              if (first) {
-                claimed |= 1u << cid;
-                ++nclaim;
-              }
+      }
+      // claim the tiles the stencil reaches: the combinations of the axes'
+      // tiles, shared out over the marker's lanes
+      int cid = 0;
+      for (int iz = 0; iz < ntl[2]; ++iz)
+        for (int iy = 0; iy < ntl[1]; ++iy)
+          for (int ix = 0; ix < ntl[0]; ++ix, ++cid) {
+            if (cid % GL != sub || !valid) continue;
+            const int tx = pick(tl[0], ix), ty = pick(tl[1], iy), tz = pick(tl[2], iz);
+            // most tiles are claimed already: an L2 read (marks only go
+            // from 0 to 1 during the gather) spares their atomic
+            uint32_t* m = a.mark + (tz * g.nty + ty) * g.ntx + tx;
+            if (__ldcg(m) == 0u && atomicExch(m, 1u) == 0u) {
+              claimed |= 1u << cid;
+              ++nclaim;
             }
-        if (a.keys && sub == 0) {
-          // the bins are valid while every stencil node lies within three
-          // cells of the home tile (the reach of the spreading's neighbour
-          // search)
-          const int t = home;
-          const int tt[3] = {t % g.ntx, (t / g.ntx) % g.nty, t / (g.ntx * g.nty)};
-          bool ok = true;
-          for (int c = 0; c < 3; ++c) {
-            const int lo = tt[c] * TILE, hi = min(lo + TILE, n3[c]) - 1;
-            ok = ok && stencil_near_home<SN>(b[c], lo, hi, n3[c], per[c]);
           }
-          if (!ok) *a.status = 1;
-        }
-    }
-      // list slots for the claimed tiles, one atomic per warp
-      int incl = nclaim;
-#pragma unroll
-      for (int off = 1; off < 32; off <<= 1) {
-        const int u = __shfl_up_sync(am, incl, off);
-        if (lane >= off) incl += u;
-    }
-      const int total = __shfl_sync(am, incl, nact - 1);
-      int base = 0;
-      if (lane == nact - 1 && total > 0) base = atomicAdd(a.nlive, total);
-      base = __shfl_sync(am, base, nact - 1) + incl - nclaim;
+      int base = claim_slots(a.nlive, nclaim, am, nact);
       if (claimed != 0u) {
         int cid2 = 0;
         for (int iz = 0; iz < ntl[2]; ++iz)
@@ -1569,21 +1718,204 @@ __device__ __forceinline__ void gather_body(const PartArgs& __restrict__ p,
                 const int tx = pick(tl[0], ix), ty = pick(tl[1], iy), tz = pick(tl[2], iz);
                 a.live_tiles[base++] = make_int4((tz * g.nty + ty) * g.ntx + tx, tx, ty, tz);
               }
-    }
+      }
     }
   }
 }
 
-template <typename S, bool WALLS, int ST, int VAR>
-__global__ void __launch_bounds__(GATHER_THREADS, (VAR == GV_LIGHT && sizeof(typename Store<S>::C) == 4) ? 6 : 4)
-gather_kernel(const PartArgs p, const GatherArgs a) {
-  gather_body<S, WALLS, ST, VAR>(p, a, blockIdx.x * (long long)blockDim.x + threadIdx.x);
+// The trilinear interpolation with eight lanes per marker (every mode; with
+// or without the node cache and the fused drift).  Lane q owns node
+// (q & 1, (q >> 1) & 1, q >> 2): its cache entry, field entry or 19
+// populations are loaded side by side with the other nodes', the node
+// velocities are added in node order through shuffles (the same sum as with
+// one lane, bit for bit), lanes 0-2 update one component of the marker each,
+// and lane q joins the hit list of one tile combination.  A launch of few
+// markers lasts as long as one marker's chain of dependent loads, which is
+// about one load per stage here (1000 markers, populations pulled: 34 us per
+// launch with one lane, whole step of the 64^3 box 66 -> 39 us).
+template <typename S, bool WALLS>
+__device__ __forceinline__ void gather_oct_body(const PartArgs& __restrict__ p,
+                                                const GatherArgs& __restrict__ a, long long gid) {
+  using C = typename Store<S>::C;
+  const Geom& g = p.g;
+  const long long M = p.M;
+  const int lane = threadIdx.x & 31;
+  const long long k = gid >> 3;
+  const int sub = lane & 7, lead = lane & ~7;
+  if (k >= M) return;                  // whole groups leave together
+  const long long wbase = gid - lane;
+  const int nact = 8 * M - wbase >= 32 ? 32 : (int)(8 * M - wbase);
+  const unsigned am = nact == 32 ? 0xffffffffu : ((1u << nact) - 1u);
+  const long long i = a.perm ? (long long)a.perm[k] : k;
+  const int n3[3] = {g.nx, g.ny, g.nz};
+  const bool per[3] = {true, true, !g.walls};
+  const int comp = sub < 3 ? sub : 2;             // the lane's component
+  int4 cb = make_int4(0, 0, 0, 0);
+  bool try_reuse = false;
+  if (a.cache == 2) {
+    cb = a.ncache_b[k];
+    try_reuse = a.invalidate == nullptr || *a.invalidate == 0;
+  }
+  const int home = a.keys ? (int)a.keys[k] : 0;
+  const bool at_aux = a.mode == GM_IBM_HALF || a.mode == GM_IBM_FINAL;
+  double X[3], vc = 0.0, im = 0.0;
+  C Fc = C(0);
+  if (a.fused) {
+    double v[3];
+    C F[3];
+    im = a.inv_mass[i];
+    drift_one<C>(p, a.drift, i, X, v, F);
+    vc = pick(v, comp);
+    if (a.include_int) Fc = pick(F, comp);
+  } else {
+    const C* fint = static_cast<const C*>(a.fint);
+    if (a.mode == GM_COUPLE) {
+      im = a.inv_mass[i];
+      vc = a.vel[comp * M + i];
+      if (a.include_int) Fc = fint[comp * M + i];
+    } else if (a.mode == GM_IBM_HALF || a.mode == GM_IBM1) {
+      Fc = fint[comp * M + i];
+    }
+    const double* P = at_aux ? a.aux : a.pos;
+#pragma unroll
+    for (int c = 0; c < 3; ++c) X[c] = P[c * M + i];
+  }
+  if (gid == 0 && a.clear_next) {      // the next step's flags (read by none now)
+    a.clear_next[0] = 0;
+    a.clear_next[1] = 0;
+  }
+  int b[3];
+  C w[3][4];
+#pragma unroll
+  for (int c = 0; c < 3; ++c) {
+    if constexpr (sizeof(C) == 4) {
+      float xh, xl;
+      split_df(X[c], xh, xl);
+      stencil_1d_df<0>(xh, xl, b[c], w[c]);
+    } else {
+      stencil_1d<0, C>(X[c], b[c], w[c]);
+    }
+  }
+  C own[3] = {C(0), C(0), C(0)};
+  if (a.mode != GM_IBM1) {
+    const int x = wrap_int(b[0] + (sub & 1), g.nx), y = wrap_int(b[1] + ((sub >> 1) & 1), g.ny);
+    int z = b[2] + (sub >> 2);
+    if (!WALLS) z = wrap_int(z, g.nz);
+    const bool in = !WALLS || (z >= 0 && z < g.nz);
+    C nv[3] = {C(0), C(0), C(0)};
+    bool reuse = false;
+    if (a.cache != 0) {
+      reuse = try_reuse && cb.x == b[0] && cb.y == b[1] && cb.z == b[2];
+      if (sub == 0 && !reuse) a.ncache_b[k] = make_int4(b[0], b[1], b[2], 0);
+    }
+    if (in) {
+      const long long cell = z * g.plane + (long long)y * g.pitch + x;
+      const int tile = tile_of(g, x, y, z);
+      C* slot = static_cast<C*>(a.ncache) + (sub * M + k) * 4;
+      C j[3], inv;
+      if (reuse) {
+        cache_load(slot, j, inv);
+      } else if (a.mom != nullptr && a.cache == 0 && a.mready[tile]) {
+        cache_load(static_cast<const C*>(a.mom) + 4 * cell, j, inv);
+      } else {
+        node_base<S, WALLS>(a, g, x, y, z, j, inv);
+        if (a.cache != 0) cache_store(slot, j, inv);
+      }
+      const C cgg[3] = {rv<C>(a.cgg[0]), rv<C>(a.cgg[1]), rv<C>(a.cgg[2])};
+      node_velocity<C>(a, cell, tile, j, inv, cgg, nv);
+    }
+    // every lane forms the whole sum, in node order
+#pragma unroll
+    for (int q = 0; q < 8; ++q) {
+      const bool node_in = !WALLS || (b[2] + (q >> 2) >= 0 && b[2] + (q >> 2) < g.nz);
+      const C wt = w[0][q & 1] * (w[1][(q >> 1) & 1] * w[2][q >> 2]);
+#pragma unroll
+      for (int c = 0; c < 3; ++c) {
+        const C u = __shfl_sync(am, nv[c], lead + q);
+        if (node_in) own[c] += wt * u;
+      }
+    }
+  }
+  // ---- the marker's update, one component per lane
+  const double s = a.s.d;
+  const C oc = pick(own, comp);
+  const int nc = pick(n3, comp);
+  const bool pc = comp < 2 || !g.walls;
+  C frec = C(0);
+  double rn = 0.0;
+  if (a.mode == GM_COUPLE) {
+    C dv[1] = {(C)vc - oc}, Fi[1] = {Fc}, zeta[1] = {C(0)}, Fh[1];
+    if (a.noise) {
+      C r[4];
+      philox_gauss4<C>((uint32_t)i, (uint32_t)(*a.tstep), 8u + (uint32_t)a.substep, 0u, a.tkey0,
+                       a.tkey1, r);
+      zeta[0] = rv<C>(a.zeta_amp) * pick(r, comp);
+    }
+    couple_force<C, 1>(a, C(im), dv, Fi, zeta, Fh);
+    const double kick = s * im;
+    const double vn = vc + kick * (double)(Fh[0] + Fc);
+    frec = -rv<C>(a.rec_weight) * Fh[0];
+    const double post_ab = sizeof(C) == 4 ? a.post_a + a.post_b : 0.0;
+    const double Xc = pick(X, comp);
+    if (a.pos_next)
+      rn = wrap_axis(sizeof(C) == 4 ? Xc + post_ab * vn : (Xc + a.post_a * vn) + a.post_b * vn, nc, pc);
+    // (the group's lanes have read the marker's state: the shuffles above)
+    if (sub < 3) {
+      a.vel[sub * M + i] = vn;
+      if (a.fh_out) static_cast<C*>(a.fh_out)[sub * M + i] = Fh[0];
+      if (a.pos_next) a.pos_next[sub * M + i] = rn;
+    }
+    if (a.pos_next && a.key_out) {
+      const double r3[3] = {__shfl_sync(am, rn, lead), __shfl_sync(am, rn, lead + 1),
+                            __shfl_sync(am, rn, lead + 2)};
+      if (sub == 0) next_bin<C>(a, g, i, r3);
+    }
+  } else if (a.mode == GM_IBM1) {
+    frec = rv<C>(a.rec_weight) * Fc;
+  } else {
+    if (sub < 3) {
+      double* out = a.mode == GM_IBM_PREDICT ? a.aux : a.pos;
+      out[sub * M + i] = wrap_axis(a.pos[sub * M + i] + s * (double)oc, nc, pc);
+    }
+    if (a.mode == GM_IBM_HALF) frec = rv<C>(a.rec_weight) * Fc;
+  }
+  if (a.rec && (a.mode == GM_COUPLE || a.mode == GM_IBM_HALF || a.mode == GM_IBM1)) {
+    const C Frec[3] = {__shfl_sync(am, frec, lead), __shfl_sync(am, frec, lead + 1),
+                       __shfl_sync(am, frec, lead + 2)};
+    if (sub == 0) {
+      write_record<0>(a, k, b, w, Frec);
+      if (a.keys && !bins_hold<2>(g, home, b)) *a.status = 1;
+    }
+    int tq[3][2];
+#pragma unroll
+    for (int c = 0; c < 3; ++c) axis_tiles<2>(b[c], w[c], n3[c], per[c], tq[c]);
+    const int tx = (sub & 1) ? tq[0][1] : tq[0][0], ty = (sub & 2) ? tq[1][1] : tq[1][0],
+              tz = (sub & 4) ? tq[2][1] : tq[2][0];
+    const int tile = (tz * g.nty + ty) * g.ntx + tx;
+    bool first = false;
+    if (tx >= 0 && ty >= 0 && tz >= 0) {
+      const uint32_t at = atomicAdd(a.hcnt + tile, 1u);
+      if (at < (uint32_t)SPREAD_HCAP) a.hits[(size_t)tile * SPREAD_HCAP + at] = (uint32_t)k;
+      first = at == 0u;
+      if (first) a.mark[tile] = 1u;
+    }
+    const unsigned m = __ballot_sync(am, first);
+    int base = 0;
+    if (lane == 0 && m != 0u) base = atomicAdd(a.nlive, __popc(m));
+    base = __shfl_sync(am, base, 0);
+    if (first) a.live_tiles[base + __popc(m & ((1u << lane) - 1u))] = make_int4(tile, tx, ty, tz);
+  }
 }
 
-
-
-
-
+template <typename S, bool WALLS, int ST, int VAR>
+__global__ void __launch_bounds__(GATHER_THREADS,
+                                  ((VAR == GV_LIGHT || VAR == GV_CACHED || VAR == GV_OCT) &&
+                                   sizeof(typename Store<S>::C) == 4) ? 6 : 4)
+gather_kernel(const PartArgs p, const GatherArgs a) {
+  const long long gid = blockIdx.x * (long long)blockDim.x + threadIdx.x;
+  if constexpr (VAR == GV_OCT) gather_oct_body<S, WALLS>(p, a, gid);
+  else gather_body<S, WALLS, ST, VAR>(p, a, gid);
+}
 
 // ------------------------------------------------------------ node moments
 // The field is filled in bricks of 32 x 4 x 4 cells (eight tiles along x):
