@@ -193,12 +193,14 @@ struct lbc_box {
   int cur;          // population array holding the current stored state
   int ia;           // force field holding F_a (pending closing-half force)
   int pc;           // particle position / velocity buffer holding the state
+  int lv;           // live-tile counter of the next record-writing gather
   bool binned;      // markers were sorted into tiles since the last set_particles
   bool steady;      // at least one step done (graphs capture steady state)
   int use_graphs;
   cudaGraphExec_t graph[2];   // two-step graphs, by starting parity of cur
   cudaGraph_t tgraph[2];      // their templates (node handles for updates)
   cudaStream_t graph_stream[2];
+  int graph_lv[2];            // lv at the capture
   // LB-kernel timing: event pairs around every LB launch (see LBC_OPT_TIMING)
   int64_t timing_cap;         // pairs available (0 = off)
   int64_t timing_used;        // pairs recorded since the last reset
@@ -545,7 +547,7 @@ struct Plan {
     a.status = b->iptr(b->L.off_status);
     a.mark = reinterpret_cast<uint32_t*>(b->arena + b->L.off_mark);
     a.live_tiles = reinterpret_cast<int4*>(b->arena + b->L.off_live);
-    a.nlive = b->iptr(b->L.off_nlive);
+    a.nlive = b->iptr(b->L.off_nlive) + b->lv;
     if (b->L.has_hits) {
       a.hcnt = reinterpret_cast<uint32_t*>(b->arena + b->L.off_hcnt);
       a.hits = reinterpret_cast<uint32_t*>(b->arena + b->L.off_hits);
@@ -603,8 +605,9 @@ struct Plan {
     a.accumulate = carry ? 1 : 0;
     a.mark = reinterpret_cast<uint32_t*>(b->arena + b->L.off_mark);
     a.live_tiles = reinterpret_cast<int4*>(b->arena + b->L.off_live);
-    a.nlive = b->iptr(b->L.off_nlive);
-    a.done = b->iptr(b->L.off_nlive) + 1;
+    a.nlive = b->iptr(b->L.off_nlive) + b->lv;
+    a.nlive_next = b->iptr(b->L.off_nlive) + (1 - b->lv);
+    b->lv = 1 - b->lv;
     if (b->L.has_hits) {
       a.hcnt = reinterpret_cast<uint32_t*>(b->arena + b->L.off_hcnt);
       a.hits = reinterpret_cast<const uint32_t*>(b->arena + b->L.off_hits);
@@ -872,7 +875,7 @@ lbc_status run_steps(lbc_box* b, int64_t nsteps, cudaStream_t s) {
   }
   if (nsteps <= 0) return LBC_OK;
   const int par = b->cur;
-  if (!b->graph[par] || b->graph_stream[par] != s) {
+  if (!b->graph[par] || b->graph_stream[par] != s || b->graph_lv[par] != b->lv) {
     if (b->graph[par]) {
       cudaGraphExecDestroy(b->graph[par]);
       b->graph[par] = nullptr;
@@ -885,7 +888,7 @@ lbc_status run_steps(lbc_box* b, int64_t nsteps, cudaStream_t s) {
       CK(cudaStreamCreateWithFlags(&cs, cudaStreamNonBlocking));
       own = true;
     }
-    const int cur0 = b->cur, ia0 = b->ia, pc0 = b->pc;
+    const int cur0 = b->cur, ia0 = b->ia, pc0 = b->pc, lv0 = b->lv;
     const bool binned0 = b->binned;
     CK(cudaStreamBeginCapture(cs, cudaStreamCaptureModeThreadLocal));
     b->capturing = true;
@@ -897,7 +900,7 @@ lbc_status run_steps(lbc_box* b, int64_t nsteps, cudaStream_t s) {
     cudaError_t e = cudaStreamEndCapture(cs, &graph);
     if (own) cudaStreamDestroy(cs);
     if (e != cudaSuccess) return LBC_ERR_CUDA;
-    if (b->cur != cur0 || b->ia != ia0 || b->pc != pc0 || b->binned != binned0) {
+    if (b->cur != cur0 || b->ia != ia0 || b->pc != pc0 || b->lv != lv0 || b->binned != binned0) {
       cudaGraphDestroy(graph);
       return LBC_ERR_STATE;
     }
@@ -926,6 +929,7 @@ lbc_status run_steps(lbc_box* b, int64_t nsteps, cudaStream_t s) {
     b->graph[par] = exec;
     b->tgraph[par] = graph;
     b->graph_stream[par] = s;
+    b->graph_lv[par] = lv0;
   }
   while (nsteps >= 2) {
     if (b->timing_cap > 0 && b->tnode[par][0]) {
@@ -1118,7 +1122,7 @@ lbc_status lbc_box_create(const lbc_lattice_desc* lat, const lbc_coupling_desc* 
   b->maxM = L.has_particles ? max_particles : 0;
   b->maxB = max_bonds;
   b->M = 0;
-  b->cur = 0; b->ia = 0; b->pc = 0;
+  b->cur = 0; b->ia = 0; b->pc = 0; b->lv = 0;
   b->binned = false; b->steady = false;
   b->use_graphs = 1;
   b->graph[0] = b->graph[1] = nullptr;
@@ -2027,10 +2031,10 @@ lbc_status batch_capture(lbc_batch* B, cudaStream_t s) {
     CK(cudaStreamCreateWithFlags(&cs, cudaStreamNonBlocking));
     own = true;
   }
-  struct Saved { int cur, ia, pc; bool binned; };
+  struct Saved { int cur, ia, pc, lv; bool binned; };
   std::vector<Saved> saved;
   for (const auto& m : B->members)
-    saved.push_back({m.box->cur, m.box->ia, m.box->pc, m.box->binned});
+    saved.push_back({m.box->cur, m.box->ia, m.box->pc, m.box->lv, m.box->binned});
   std::vector<BoxEntry> host[2];
   std::vector<PartEntry> phost[2];
   int64_t l = 0;
@@ -2047,7 +2051,7 @@ lbc_status batch_capture(lbc_batch* B, cudaStream_t s) {
   for (size_t j = 0; j < B->members.size(); ++j) {
     const lbc_box* b = B->members[j].box;
     const Saved& v = saved[j];
-    if (b->cur != v.cur || b->ia != v.ia || b->pc != v.pc || b->binned != v.binned) {
+    if (b->cur != v.cur || b->ia != v.ia || b->pc != v.pc || b->lv != v.lv || b->binned != v.binned) {
       cudaGraphDestroy(graph);
       return LBC_ERR_STATE;
     }

@@ -120,6 +120,17 @@ struct alignas(16) StencilRecT {
   C pad;
 };
 
+// the trilinear record: packed base (pack_base), the weight of the upper node
+// per axis (the lower node's is 1 - t) and the force to spread: 32 bytes for
+// float, one sector
+template <typename C>
+struct alignas(16) TriRecT {
+  unsigned long long base;
+  C t[3];
+  C F[3];
+};
+static_assert(sizeof(TriRecT<float>) == 32 && sizeof(TriRecT<double>) == 64, "");
+
 // bytes of one force-field element and of one stencil record
 inline size_t force_elem_bytes(int storage) { return storage == ST_F64 ? 8 : 4; }
 inline size_t stencil_rec_bytes(int storage) {
@@ -265,8 +276,8 @@ struct GatherArgs {
   const void* fint;               // [3][M] intrinsic forces, compute type
   const double* inv_mass;
   void* fh_out;                   // [3][M] coupling force F^h, compute type
-  void* rec;                      // StencilRecT<C>[M], by sorted slot
-  unsigned long long* reach;      // stencil base per sorted slot (pack_base)
+  void* rec;                      // TriRecT<C>[M] (trilinear) or StencilRecT<C>[M], by sorted slot
+  unsigned long long* reach;      // 4- and 3-point: stencil base per sorted slot (pack_base)
   int* status;                    // set to 1 if a marker left its home tile +- 1 cell
   // tiles a stencil reaches: mark[t] is set once per tile and the tile is
   // appended to live_tiles[0 .. *nlive) for the spreading that follows
@@ -306,8 +317,8 @@ void launch_node_moments(const PartArgs& p, const GatherArgs& a, const int2* bri
 constexpr int SPREAD_HCAP = 32;
 
 struct SpreadArgs {
-  const void* rec;                            // StencilRecT<C>[M]
-  const unsigned long long* reach;            // stencil base per sorted slot (pack_base)
+  const void* rec;                            // the gather's records
+  const unsigned long long* reach;            // 4- and 3-point: stencil bases
   const int* tile_begin; const int* tile_end;
   // per axis and tile, the (up to 8) tiles holding markers whose stencil can
   // reach it: ntab[(axis * maxnt + t) * 8 + q], -1 padded
@@ -316,11 +327,11 @@ struct SpreadArgs {
   int accumulate;                 // 1: add onto the tiles whose flag is set
   uint32_t* mark;                 // marks of the gather; consumed here
   const int4* live_tiles;         // the marked tiles (t, tx, ty, tz), in any order
-  int* nlive;                     // their count; reset to 0 on exit
+  const int* nlive;               // their count
+  int* nlive_next;                // the next gather's counter, zeroed here (two take turns)
   // the gather's hit lists (null: off); a tile's count is reset to 0 when
   // it is spread, and a list longer than SPREAD_HCAP takes the search
   uint32_t* hcnt; const uint32_t* hits;
-  int* done;                      // blocks finished (reset to 0 on exit)
 };
 // host: fill the neighbour-tile table (3 * maxnt * 4 ints)
 void neighbour_tiles(const Geom& g, int maxnt, int* table);

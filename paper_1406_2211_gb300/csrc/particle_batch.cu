@@ -104,7 +104,7 @@ gather_batch_kernel(const PartEntry* __restrict__ tab, int n) {
 }
 
 template <int ST>
-__global__ void __launch_bounds__(SPREAD_THREADS, 4)
+__global__ void __launch_bounds__(SPREAD_THREADS, SPREAD_RESIDENT)
 spread_batch_kernel(const PartEntry* __restrict__ tab, int n) {
   __shared__ SharedEntry<HEAD + U_SPREAD> se;
   const PartEntry& e = stage<U_SPREAD>(tab, n, se);

@@ -1119,18 +1119,27 @@ __device__ __forceinline__ void next_bin(const GatherArgs& a, const Geom& g, lon
   if (a.home && !(F32 ? near_home_f(g, a.home[i], rn) : near_home(g, a.home[i], rn))) *a.need_next = 1;
 }
 
-// the stencil record of slot k and its packed base
+// the spreading's record of slot k (and its packed base)
 template <int ST, typename C>
-__device__ __forceinline__ void write_record(const GatherArgs& a, long long k, const int (&b)[3],
+__device__ __forceinline__ void write_record(const GatherArgs& a, const Geom& g, long long k, const int (&b)[3],
                                              const C (&w)[3][4], const C (&F)[3]) {
-  StencilRecT<C> r;
-  r.bx = b[0]; r.by = b[1]; r.bz = b[2]; r.kind = ST;
+  if constexpr (ST == 0) {
+    TriRecT<C> r;
+    // (periodic coordinates wrapped into the box)
+    r.base = pack_base(wrap_int(b[0], g.nx), wrap_int(b[1], g.ny), g.walls ? b[2] : wrap_int(b[2], g.nz));
 #pragma unroll
-  for (int q = 0; q < 4; ++q) { r.wx[q] = w[0][q]; r.wy[q] = w[1][q]; r.wz[q] = w[2][q]; }
-  r.F[0] = F[0]; r.F[1] = F[1]; r.F[2] = F[2];
-  r.pad = C(0);
-  static_cast<StencilRecT<C>*>(a.rec)[k] = r;
-  a.reach[k] = pack_base(b[0], b[1], b[2]);
+    for (int c = 0; c < 3; ++c) { r.t[c] = w[c][1]; r.F[c] = F[c]; }
+    static_cast<TriRecT<C>*>(a.rec)[k] = r;
+  } else {
+    StencilRecT<C> r;
+    r.bx = b[0]; r.by = b[1]; r.bz = b[2]; r.kind = ST;
+#pragma unroll
+    for (int q = 0; q < 4; ++q) { r.wx[q] = w[0][q]; r.wy[q] = w[1][q]; r.wz[q] = w[2][q]; }
+    r.F[0] = F[0]; r.F[1] = F[1]; r.F[2] = F[2];
+    r.pad = C(0);
+    static_cast<StencilRecT<C>*>(a.rec)[k] = r;
+    a.reach[k] = pack_base(b[0], b[1], b[2]);
+  }
 }
 
 // v[q] by selects (the array stays in registers)
@@ -1625,7 +1634,7 @@ __device__ __forceinline__ void gather_body(const PartArgs& __restrict__ p,
   }
   if (a.rec && (a.mode == GM_COUPLE || a.mode == GM_IBM_HALF || a.mode == GM_IBM1)) {
     if (sub == 0 && valid) {
-      write_record<ST>(a, k, b, w, Frec);
+      write_record<ST>(a, g, k, b, w, Frec);
       if (a.keys && !bins_hold<SN>(g, home, b)) *a.status = 1;
     }
     if constexpr (SN == 2) {
@@ -1883,7 +1892,7 @@ __device__ __forceinline__ void gather_oct_body(const PartArgs& __restrict__ p,
     const C Frec[3] = {__shfl_sync(am, frec, lead), __shfl_sync(am, frec, lead + 1),
                        __shfl_sync(am, frec, lead + 2)};
     if (sub == 0) {
-      write_record<0>(a, k, b, w, Frec);
+      write_record<0>(a, g, k, b, w, Frec);
       if (a.keys && !bins_hold<2>(g, home, b)) *a.status = 1;
     }
     int tq[3][2];
@@ -2087,302 +2096,476 @@ __device__ inline void tile_weights_shift(int e, const C (&w)[4], C (&out)[TILE]
   }
 }
 
-// a surviving marker reduced to the current tile: per axis the weights at
-// the tile's TILE cells, and its force
+// a surviving marker reduced to the current tile: the weights at the tile's
+// TILE cells of each axis and its force, each component twice (FP32: the
+// operand pairs of the packed multiply-adds).  The z weights stand in the
+// order 0, 2, 1, 3: a lane owns the cells z, z + 2.
 template <typename C>
-struct SpreadHit {
-  C w[3][TILE];
-  C F[3];
-  C pad;
+struct alignas(16) SpreadHit {
+  C wx[TILE], wy[TILE], wz[TILE];
+  C F[sizeof(C) == 4 ? 8 : 4];
 };
 
-constexpr int SPREAD_THREADS = 256;
-constexpr int SPREAD_ROUNDS = 4;     // candidate rounds of 32 whose loads are in flight together
+__device__ __forceinline__ void put4(float* p, float a, float b, float c, float d) {
+  *reinterpret_cast<float4*>(p) = make_float4(a, b, c, d);
+}
+__device__ __forceinline__ void put4(double* p, double a, double b, double c, double d) {
+  reinterpret_cast<double2*>(p)[0] = make_double2(a, b);
+  reinterpret_cast<double2*>(p)[1] = make_double2(c, d);
+}
 
-// Spreading, one warp per live tile (a tile some stencil reaches), taken from
-// the list the gather built.  Lane l owns the cells (l & 3, (l >> 2) & 3,
-// l >> 4) and the same cell two planes up, and keeps their force sums in
-// registers.  The candidates are the markers binned in the neighbour tiles;
-// 32 of them are tested at a time, each surviving lane reduces its own
-// marker to the tile, and the warp then adds the survivors in candidate
-// order, so the sums are formed in a fixed order (no atomics).
-// the body of the spreading for block bid of nblk blocks of one box
-template <int ST, typename C>
-__device__ __forceinline__ void spread_body(const PartArgs& __restrict__ p,
-                                            const SpreadArgs& __restrict__ a, int bid, int nblk) {
-  static_assert(TILE == 4 && TILE_CELLS == 64, "two cells per lane");
-  constexpr int SN = nodes_1d<ST>();
-  constexpr int WARPS = SPREAD_THREADS / 32;
-  __shared__ SpreadHit<C> shit[WARPS][32];
-  __shared__ int shk[WARPS][32 * SPREAD_ROUNDS];   // hits of a candidate group, in order
-  const Geom& g = p.g;
-  const int lane = threadIdx.x & 31, wid = threadIdx.x >> 5;
-  SpreadHit<C>* stage = shit[wid];
-  int* hk = shk[wid];
-  const StencilRecT<C>* recs = static_cast<const StencilRecT<C>*>(a.rec);
-  C* F = static_cast<C*>(a.F);
-  const int ntiles = g.ntx * g.nty * g.ntz;
-  const bool perz = !g.walls;
-  // tiles no stencil reaches keep their flag when accumulating and are
-  // cleared otherwise; the marks are consumed (the live tiles are other
-  // tiles, so the warps go on without waiting for each other)
-  {
-    // four tiles per thread and access (marks and flags start 256-byte
-    // aligned), the remainder one by one
-    const long long gt = (long long)bid * blockDim.x + threadIdx.x;
-    const long long nthreads = (long long)nblk * blockDim.x;
-    const long long n4 = ntiles / 4;
-    uint4* mark4 = reinterpret_cast<uint4*>(a.mark);
-    uchar4* flag4 = reinterpret_cast<uchar4*>(a.flag);
-    for (long long q = gt; q < n4; q += nthreads) {
-      const uint4 m = mark4[q];
-      const bool any = (m.x | m.y | m.z | m.w) != 0u;
-      if (any) mark4[q] = make_uint4(0u, 0u, 0u, 0u);
-      if (!a.accumulate) {
-        if (!any) {
-          flag4[q] = make_uchar4(0, 0, 0, 0);
-        } else {
-          // a live tile's flag is set by the warp that spreads it: only
-          // the other flags are written
-          uint8_t* f = a.flag + 4 * q;
-          if (!m.x) f[0] = 0;
-          if (!m.y) f[1] = 0;
-          if (!m.z) f[2] = 0;
-          if (!m.w) f[3] = 0;
-        }
-      }
-    }
-    for (long long t = 4 * n4 + gt; t < ntiles; t += nthreads) {
-      if (a.mark[t] != 0u) a.mark[t] = 0u;
-      else if (!a.accumulate) a.flag[t] = 0;
+// reduces one marker (base b, per-axis weights w, force F) to the tile at lo
+template <int SN, typename C>
+__device__ __forceinline__ void reduce_hit(SpreadHit<C>& h, const Geom& g, const int (&b)[3],
+                                           const C (&w)[3][4], const C (&F)[3], const int (&lo)[3]) {
+  const int n3[3] = {g.nx, g.ny, g.nz};
+#pragma unroll
+  for (int d = 0; d < 3; ++d) {
+    const bool periodic = d < 2 || !g.walls;
+    C wt[TILE];
+    // (axes on which a stencil meets a tile only by shifting: see tile_offset)
+    if (!periodic || n3[d] >= 2 * TILE)
+      tile_weights_shift<SN, C>(tile_offset(b[d], lo[d], n3[d], periodic), w[d], wt);
+    else
+      tile_weights<SN, C>(b[d], w[d], n3[d], periodic, lo[d], wt);
+#pragma unroll
+    for (int j = 0; j < TILE; ++j) {
+      if (d == 0) h.wx[j] = wt[j];
+      else if (d == 1) h.wy[j] = wt[j];
+      else h.wz[(j & 1) * 2 + (j >> 1)] = wt[j];
     }
   }
-  const int nlive = __shfl_sync(0xffffffffu, lane == 0 ? *a.nlive : 0, 0);
-  const int cxl = lane & 3, cyl = (lane >> 2) & 3, czl = lane >> 4;
-  // axes on which a stencil meets a tile only by shifting (see tile_offset)
-  const bool shx = g.nx >= 2 * TILE, shy = g.ny >= 2 * TILE, shz = !perz || g.nz >= 2 * TILE;
-  // axes of whole tiles: the neighbour tiles are t - 1, t, t + 1 (wrapped, or
-  // clipped at walls), the same list the table holds
-  const int n3[3] = {g.nx, g.ny, g.nz}, ntv[3] = {g.ntx, g.nty, g.ntz};
-  bool whole[3];
 #pragma unroll
-  for (int d = 0; d < 3; ++d)
-    whole[d] = n3[d] % TILE == 0 && (!(d < 2 || perz) || ntv[d] >= 3);
-  const int stride = nblk * WARPS;
-  int j = bid * WARPS + wid;
-  // software pipeline over the warp's tiles: the list entry two tiles
-  // ahead, and the hit list (count and entries) of the next tile, are
-  // loaded while this one is spread
-  int4 lt_next = j < nlive ? a.live_tiles[j] : make_int4(0, 0, 0, 0);
-  int4 lt_next2 = j + stride < nlive ? a.live_tiles[j + stride] : make_int4(0, 0, 0, 0);
-  uint32_t hc_next = 0u, key_next = 0u;
-  if (a.hcnt != nullptr && j < nlive) {
-    hc_next = a.hcnt[lt_next.x];
-    key_next = a.hits[(size_t)lt_next.x * SPREAD_HCAP + lane];
-  }
-  for (; j < nlive; j += stride) {
-    const int4 lt = lt_next;
-    const uint32_t hc_cur = hc_next, key_cur = key_next;
-    lt_next = lt_next2;
-    if (j + 2 * stride < nlive) lt_next2 = a.live_tiles[j + 2 * stride];
-    if (a.hcnt != nullptr && j + stride < nlive) {
-      hc_next = a.hcnt[lt_next.x];
-      key_next = a.hits[(size_t)lt_next.x * SPREAD_HCAP + lane];
-    }
-    const int t = lt.x;
-    const int tt[3] = {lt.y, lt.z, lt.w};
-    const int lo[3] = {tt[0] * TILE, tt[1] * TILE, tt[2] * TILE};
-    const int hi[3] = {min(lo[0] + TILE, g.nx) - 1, min(lo[1] + TILE, g.ny) - 1, min(lo[2] + TILE, g.nz) - 1};
-    const int x = lo[0] + cxl, y = lo[1] + cyl, z0 = lo[2] + czl, z1 = z0 + 2;
-    const bool in0 = x <= hi[0] && y <= hi[1] && z0 <= hi[2];
-    const bool in1 = x <= hi[0] && y <= hi[1] && z1 <= hi[2];
-    const long long cell0 = z0 * g.plane + (long long)y * g.pitch + x;
-    const long long cell1 = cell0 + 2 * g.plane;
-    C acc0[3] = {C(0), C(0), C(0)}, acc1[3] = {C(0), C(0), C(0)};
-    if (a.accumulate && a.flag[t]) {
-      if (in0) load_force(F, cell0, acc0[0], acc0[1], acc0[2]);
-      if (in1) load_force(F, cell1, acc1[0], acc1[1], acc1[2]);
-    }
-    // adds the markers listed in hk[0 .. nhit), in that order
-    auto add_hits = [&](int nhit) {
-      for (int hb = 0; hb < nhit; hb += 32) {
-        const int nh = min(32, nhit - hb);
-        if (lane < nh) {
-          const StencilRecT<C>& r = recs[hk[hb + lane]];
-          SpreadHit<C>& h = stage[lane];
-          int e[3];
-          e[0] = tile_offset(r.bx, lo[0], g.nx, true);
-          e[1] = tile_offset(r.by, lo[1], g.ny, true);
-          e[2] = tile_offset(r.bz, lo[2], g.nz, perz);
-          C rw[4];
-#pragma unroll
-          for (int q2 = 0; q2 < 4; ++q2) rw[q2] = r.wx[q2];
-          if (shx) tile_weights_shift<SN, C>(e[0], rw, h.w[0]);
-          else tile_weights<SN, C>(r.bx, rw, g.nx, true, lo[0], h.w[0]);
-#pragma unroll
-          for (int q2 = 0; q2 < 4; ++q2) rw[q2] = r.wy[q2];
-          if (shy) tile_weights_shift<SN, C>(e[1], rw, h.w[1]);
-          else tile_weights<SN, C>(r.by, rw, g.ny, true, lo[1], h.w[1]);
-#pragma unroll
-          for (int q2 = 0; q2 < 4; ++q2) rw[q2] = r.wz[q2];
-          if (shz) tile_weights_shift<SN, C>(e[2], rw, h.w[2]);
-          else tile_weights<SN, C>(r.bz, rw, g.nz, perz, lo[2], h.w[2]);
-          h.F[0] = r.F[0]; h.F[1] = r.F[1]; h.F[2] = r.F[2];
-        }
-        __syncwarp();
-        for (int src = 0; src < nh; ++src) {
-          const SpreadHit<C>& h = stage[src];
-          const C wxy = h.w[0][cxl] * h.w[1][cyl];
-          const C w0 = wxy * h.w[2][czl], w1 = wxy * h.w[2][czl + 2];
-          const C f0 = h.F[0], f1 = h.F[1], f2 = h.F[2];
-          acc0[0] += w0 * f0; acc0[1] += w0 * f1; acc0[2] += w0 * f2;
-          acc1[0] += w1 * f0; acc1[1] += w1 * f1; acc1[2] += w1 * f2;
-        }
-        __syncwarp();
-      }
-    };
-    // hit list of the tile, built by the gather (trilinear stencils): the
-    // markers whose stencil reaches it, sorted by slot so the sums run in a
-    // fixed order; a list that overflowed (or none) takes the search below
-    int hc = SPREAD_HCAP + 1;
-    if (a.hcnt != nullptr) {
-      hc = (int)hc_cur;
-      uint32_t key = key_cur;
-      if (hc <= SPREAD_HCAP) {
-        if (lane >= hc) key = 0xFFFFFFFFu;
-#pragma unroll
-        for (int kk2 = 2; kk2 <= 32; kk2 <<= 1)
-#pragma unroll
-          for (int jj = kk2 >> 1; jj > 0; jj >>= 1) {
-            const uint32_t other = __shfl_xor_sync(0xffffffffu, key, jj);
-            const bool lower = (lane & jj) == 0, up = (lane & kk2) == 0;
-            key = lower == up ? min(key, other) : max(key, other);
-          }
-        if (lane < hc) hk[lane] = (int)key;
-        __syncwarp();
-        add_hits(hc);
-      }
-      __syncwarp();
-      if (lane == 0) a.hcnt[t] = 0u;           // empty for the next gather
-    }
-    if (hc > SPREAD_HCAP) {
-    // neighbour tiles per axis: lane q holds entry q of the list (from the
-    // table on axes of partial or few tiles)
-    int rowv[3], nt[3];
-#pragma unroll
-    for (int d = 0; d < 3; ++d) {
-      if (whole[d]) {
-        const bool periodic = d < 2 || perz;
-        const int first = periodic ? tt[d] - 1 : max(tt[d] - 1, 0);
-        const int last = periodic ? tt[d] + 1 : min(tt[d] + 1, ntv[d] - 1);
-        nt[d] = last - first + 1;
-        int v = first + lane;
-        if (v < 0) v += ntv[d];
-        else if (v >= ntv[d]) v -= ntv[d];
-        rowv[d] = lane < nt[d] ? v : -1;
-      } else {
-        const int* row = a.ntab + (d * a.maxnt + tt[d]) * MAXNT;
-        rowv[d] = lane < MAXNT ? row[lane] : -1;
-        nt[d] = __popc(__ballot_sync(0xffffffffu, rowv[d] >= 0));
-      }
-    }
-    const int ncand = nt[0] * nt[1] * nt[2];
-    // candidate markers: the ranges of the neighbour tiles, flattened; 32
-    // neighbour tiles per chunk (one load each), then the candidates in
-    // groups of SPREAD_ROUNDS x 32: their reach loads are all issued before
-    // any is tested, the hits of the group are listed in candidate order in
-    // shared memory, and their stencil records are loaded 32 at a time with
-    // one load per lane.  The hits are added in candidate order (markers
-    // sorted by tile, neighbour tiles in a fixed order), so the sums do not
-    // depend on scheduling.
-    for (int qbase = 0; qbase < ncand; qbase += 32) {
-      const int q = qbase + lane;
-      int qx, qy, qz;
-      if (nt[0] == 3 && nt[1] == 3) {    // the usual 3 x 3 x 3 neighbourhood
-        qx = q % 3; qy = (q / 3) % 3; qz = (q / 9) & (MAXNT - 1);
-      } else {
-        qx = q % nt[0]; qy = (q / nt[0]) % nt[1]; qz = (q / (nt[0] * nt[1])) & (MAXNT - 1);
-      }
-      const int tx = __shfl_sync(0xffffffffu, rowv[0], qx);
-      const int ty = __shfl_sync(0xffffffffu, rowv[1], qy);
-      const int tz = __shfl_sync(0xffffffffu, rowv[2], qz);
-      int cnt = 0, kb = 0;
-      if (q < ncand) {
-        const int tn = (tz * g.nty + ty) * g.ntx + tx;
-        kb = a.tile_begin[tn];
-        cnt = a.tile_end[tn] - kb;
-      }
-      int incl = cnt;                    // inclusive prefix of the counts
-      for (int off = 1; off < 32; off <<= 1) {
-        const int v = __shfl_up_sync(0xffffffffu, incl, off);
-        if (lane >= off) incl += v;
-      }
-      const int total = __shfl_sync(0xffffffffu, incl, 31);
-      for (int cbase = 0; cbase < total; cbase += 32 * SPREAD_ROUNDS) {
-        int kk[SPREAD_ROUNDS];
-        unsigned long long rr[SPREAD_ROUNDS];
-#pragma unroll
-        for (int r = 0; r < SPREAD_ROUNDS; ++r) {
-          kk[r] = -1;
-          rr[r] = 0ull;
-          if (cbase + 32 * r >= total) continue;     // warp-uniform: no candidates left
-          const int cidx = cbase + 32 * r + lane;
-          // owning chunk lane: the first lane whose inclusive prefix exceeds cidx
-          int pos = 0;
-#pragma unroll
-          for (int step = 16; step > 0; step >>= 1) {
-            const int v = __shfl_sync(0xffffffffu, incl, pos + step - 1);
-            if (v <= cidx) pos += step;
-          }
-          const int ex = __shfl_sync(0xffffffffu, incl - cnt, pos);
-          const int kq = __shfl_sync(0xffffffffu, kb, pos);
-          kk[r] = cidx < total ? kq + (cidx - ex) : -1;
-          if (kk[r] >= 0) rr[r] = a.reach[kk[r]];
-        }
-        int nhit = 0;
-#pragma unroll
-        for (int r = 0; r < SPREAD_ROUNDS; ++r) {
-          if (cbase + 32 * r >= total) break;       // warp-uniform
-          bool hit = false;
-          if (kk[r] >= 0) {
-            const int rvx = base_x(rr[r]), rvy = base_y(rr[r]), rvz = base_z(rr[r]);
-            const int e0 = tile_offset(rvx, lo[0], g.nx, true);
-            const int e1 = tile_offset(rvy, lo[1], g.ny, true);
-            const int e2 = tile_offset(rvz, lo[2], g.nz, perz);
-            hit = (shx ? e0 <= hi[0] - lo[0] && e0 + SN - 1 >= 0
-                       : axis_reach<SN>(rvx, g.nx, true, lo[0], hi[0])) &&
-                  (shy ? e1 <= hi[1] - lo[1] && e1 + SN - 1 >= 0
-                       : axis_reach<SN>(rvy, g.ny, true, lo[1], hi[1])) &&
-                  (shz ? e2 <= hi[2] - lo[2] && e2 + SN - 1 >= 0
-                       : axis_reach<SN>(rvz, g.nz, perz, lo[2], hi[2]));
-          }
-          const unsigned m = __ballot_sync(0xffffffffu, hit);
-          if (hit) hk[nhit + __popc(m & ((1u << lane) - 1u))] = kk[r];
-          nhit += __popc(m);
-        }
-        __syncwarp();
-        add_hits(nhit);
-      }
-    }
-    }
-    if (in0) store_force(F, cell0, acc0[0], acc0[1], acc0[2]);
-    if (in1) store_force(F, cell1, acc1[0], acc1[1], acc1[2]);
-    if (lane == 0) a.flag[t] = 1;
-  }
-  // the last block to finish resets the list for the next gather (every
-  // block read the count before it got here)
-  __syncthreads();
-  if (threadIdx.x == 0) {
-    __threadfence();
-    if (atomicAdd(a.done, 1) == nblk - 1) {
-      *a.nlive = 0;
-      *a.done = 0;
-    }
+  for (int c = 0; c < 3; ++c) {
+    if (sizeof(C) == 4) h.F[2 * c] = h.F[2 * c + 1] = F[c];
+    else h.F[c] = F[c];
   }
 }
 
+// the same from the record of a slot
 template <int ST, typename C>
-__global__ void __launch_bounds__(SPREAD_THREADS, 4)
+__device__ __forceinline__ void reduce_record(SpreadHit<C>& h, const Geom& g, const SpreadArgs& a,
+                                              int slot, const int (&lo)[3]) {
+  C w[3][4], F[3];
+  int b[3];
+  if constexpr (ST == 0) {
+    const TriRecT<C> r = static_cast<const TriRecT<C>*>(a.rec)[slot];
+    b[0] = base_x(r.base); b[1] = base_y(r.base); b[2] = base_z(r.base);
+#pragma unroll
+    for (int d = 0; d < 3; ++d) {
+      w[d][0] = C(1) - r.t[d]; w[d][1] = r.t[d]; w[d][2] = w[d][3] = C(0);
+      F[d] = r.F[d];
+    }
+  } else {
+    const StencilRecT<C>& r = static_cast<const StencilRecT<C>*>(a.rec)[slot];
+    b[0] = r.bx; b[1] = r.by; b[2] = r.bz;
+#pragma unroll
+    for (int q = 0; q < 4; ++q) { w[0][q] = r.wx[q]; w[1][q] = r.wy[q]; w[2][q] = r.wz[q]; }
+#pragma unroll
+    for (int d = 0; d < 3; ++d) F[d] = r.F[d];
+  }
+  reduce_hit<nodes_1d<ST>(), C>(h, g, b, w, F, lo);
+}
+
+// A lane's force sums at its cells z and z + 2: a[c] += (wx wy wz) F_c.  FP32
+// takes both cells with one paired multiply-add (the same rounding as two
+// single ones).
+template <typename C>
+struct TileSum {
+  C a[3][2];
+  __device__ void zero() {
+#pragma unroll
+    for (int c = 0; c < 3; ++c) a[c][0] = a[c][1] = C(0);
+  }
+  __device__ void add(const SpreadHit<C>& h, int cx, int cy, int cz) {
+    const C wxy = h.wx[cx] * h.wy[cy];
+    if constexpr (sizeof(C) == 4) {
+      const float4 f01 = *reinterpret_cast<const float4*>(&h.F[0]);
+      const float2 f2 = *reinterpret_cast<const float2*>(&h.F[4]);
+      const float2 f[3] = {make_float2(f01.x, f01.y), make_float2(f01.z, f01.w), f2};
+      const float2 w = __fmul2_rn(make_float2(wxy, wxy), *reinterpret_cast<const float2*>(&h.wz[2 * cz]));
+#pragma unroll
+      for (int c = 0; c < 3; ++c) {
+        const float2 r = __ffma2_rn(w, f[c], make_float2(a[c][0], a[c][1]));
+        a[c][0] = r.x;
+        a[c][1] = r.y;
+      }
+    } else {
+#pragma unroll
+      for (int q = 0; q < 2; ++q) {
+        const C w = wxy * h.wz[2 * cz + q];
+#pragma unroll
+        for (int c = 0; c < 3; ++c) a[c][q] += w * h.F[c];
+      }
+    }
+  }
+};
+
+constexpr int SPREAD_THREADS = 256;
+constexpr int SPREAD_WARPS = SPREAD_THREADS / 32;
+constexpr int SPREAD_ROUNDS = 4;     // candidate rounds of 32 whose loads are in flight together
+
+// One live tile t (index, tx, ty, tz) by a whole warp, its markers found by a
+// search of the markers binned in the neighbour tiles.  Lane l owns the cells
+// (l & 3, (l >> 2) & 3, l >> 4) and the same cell two planes up, and keeps
+// their force sums in registers; 32 candidates are tested at a time, each
+// surviving lane reduces its own marker to the tile, and the warp then adds
+// the survivors in candidate order, so the sums are formed in a fixed order
+// (no atomics).  stage: 32 hits, hk: 32 SPREAD_ROUNDS slots of this warp.
+template <int ST, typename C>
+__device__ __forceinline__ void spread_search_tile(const Geom& g, const SpreadArgs& a, const int4& t,
+                                                   SpreadHit<C>* stage, int* hk) {
+  constexpr int SN = nodes_1d<ST>();
+  constexpr unsigned full = 0xffffffffu;
+  const int lane = threadIdx.x & 31;
+  const int cxl = lane & 3, cyl = (lane >> 2) & 3, czl = lane >> 4;
+  const bool perz = !g.walls;
+  C* F = static_cast<C*>(a.F);
+  const int lo[3] = {t.y * TILE, t.z * TILE, t.w * TILE};
+  const int hi[3] = {min(lo[0] + TILE, g.nx) - 1, min(lo[1] + TILE, g.ny) - 1, min(lo[2] + TILE, g.nz) - 1};
+  const int x = lo[0] + cxl, y = lo[1] + cyl, z0 = lo[2] + czl;
+  const bool in0 = x <= hi[0] && y <= hi[1] && z0 <= hi[2];
+  const bool in1 = x <= hi[0] && y <= hi[1] && z0 + 2 <= hi[2];
+  const long long cell0 = z0 * g.plane + (long long)y * g.pitch + x;
+  const long long cell1 = cell0 + 2 * g.plane;
+  TileSum<C> sum;
+  sum.zero();
+  if (a.accumulate && a.flag[t.x]) {
+    if (in0) load_force(F, cell0, sum.a[0][0], sum.a[1][0], sum.a[2][0]);
+    if (in1) load_force(F, cell1, sum.a[0][1], sum.a[1][1], sum.a[2][1]);
+  }
+  // axes on which a stencil meets a tile only by shifting (see tile_offset)
+  const bool shx = g.nx >= 2 * TILE, shy = g.ny >= 2 * TILE, shz = !perz || g.nz >= 2 * TILE;
+  // axes of whole tiles: the neighbour tiles are t - 1, t, t + 1 (wrapped,
+  // or clipped at walls), the same list the table holds
+  const int n3[3] = {g.nx, g.ny, g.nz}, ntv[3] = {g.ntx, g.nty, g.ntz};
+  const int tt[3] = {t.y, t.z, t.w};
+  // neighbour tiles per axis: lane q holds entry q of the list (from the
+  // table on axes of partial or few tiles)
+  int rowv[3], nt[3];
+#pragma unroll
+  for (int d = 0; d < 3; ++d) {
+    const bool periodic = d < 2 || perz;
+    if (n3[d] % TILE == 0 && (!periodic || ntv[d] >= 3)) {
+      const int first = periodic ? tt[d] - 1 : max(tt[d] - 1, 0);
+      const int last = periodic ? tt[d] + 1 : min(tt[d] + 1, ntv[d] - 1);
+      nt[d] = last - first + 1;
+      int v = first + lane;
+      if (v < 0) v += ntv[d];
+      else if (v >= ntv[d]) v -= ntv[d];
+      rowv[d] = lane < nt[d] ? v : -1;
+    } else {
+      const int* row = a.ntab + (d * a.maxnt + tt[d]) * MAXNT;
+      rowv[d] = lane < MAXNT ? row[lane] : -1;
+      nt[d] = __popc(__ballot_sync(full, rowv[d] >= 0));
+    }
+  }
+  const int ncand = nt[0] * nt[1] * nt[2];
+  // candidate markers: the ranges of the neighbour tiles, flattened; 32
+  // neighbour tiles per chunk (one load each), then the candidates in
+  // groups of SPREAD_ROUNDS x 32: their reach loads are all issued before
+  // any is tested, the hits of the group are listed in candidate order in
+  // shared memory, and their stencil records are loaded 32 at a time with
+  // one load per lane.  The hits are added in candidate order (markers
+  // sorted by tile, neighbour tiles in a fixed order), so the sums do not
+  // depend on scheduling.
+  for (int qbase = 0; qbase < ncand; qbase += 32) {
+    const int q = qbase + lane;
+    int qx, qy, qz;
+    if (nt[0] == 3 && nt[1] == 3) {    // the usual 3 x 3 x 3 neighbourhood
+      qx = q % 3; qy = (q / 3) % 3; qz = (q / 9) & (MAXNT - 1);
+    } else {
+      qx = q % nt[0]; qy = (q / nt[0]) % nt[1]; qz = (q / (nt[0] * nt[1])) & (MAXNT - 1);
+    }
+    const int tx = __shfl_sync(full, rowv[0], qx);
+    const int ty = __shfl_sync(full, rowv[1], qy);
+    const int tz = __shfl_sync(full, rowv[2], qz);
+    int cnt = 0, kb = 0;
+    if (q < ncand) {
+      const int tn = (tz * g.nty + ty) * g.ntx + tx;
+      kb = a.tile_begin[tn];
+      cnt = a.tile_end[tn] - kb;
+    }
+    int incl = cnt;                    // inclusive prefix of the counts
+    for (int off = 1; off < 32; off <<= 1) {
+      const int v = __shfl_up_sync(full, incl, off);
+      if (lane >= off) incl += v;
+    }
+    const int total = __shfl_sync(full, incl, 31);
+    for (int cbase = 0; cbase < total; cbase += 32 * SPREAD_ROUNDS) {
+      int kk[SPREAD_ROUNDS];
+      unsigned long long rr[SPREAD_ROUNDS];
+#pragma unroll
+      for (int r = 0; r < SPREAD_ROUNDS; ++r) {
+        kk[r] = -1;
+        rr[r] = 0ull;
+        if (cbase + 32 * r >= total) continue;     // warp-uniform: no candidates left
+        const int cidx = cbase + 32 * r + lane;
+        // owning chunk lane: the first lane whose inclusive prefix exceeds cidx
+        int pos = 0;
+#pragma unroll
+        for (int step = 16; step > 0; step >>= 1) {
+          const int v = __shfl_sync(full, incl, pos + step - 1);
+          if (v <= cidx) pos += step;
+        }
+        const int ex = __shfl_sync(full, incl - cnt, pos);
+        const int kq = __shfl_sync(full, kb, pos);
+        kk[r] = cidx < total ? kq + (cidx - ex) : -1;
+        if (kk[r] >= 0) {
+          if constexpr (ST == 0) rr[r] = static_cast<const TriRecT<C>*>(a.rec)[kk[r]].base;
+          else rr[r] = a.reach[kk[r]];
+        }
+      }
+      int nhit = 0;
+#pragma unroll
+      for (int r = 0; r < SPREAD_ROUNDS; ++r) {
+        if (cbase + 32 * r >= total) break;       // warp-uniform
+        bool hit = false;
+        if (kk[r] >= 0) {
+          const int rvx = base_x(rr[r]), rvy = base_y(rr[r]), rvz = base_z(rr[r]);
+          const int e0 = tile_offset(rvx, lo[0], g.nx, true);
+          const int e1 = tile_offset(rvy, lo[1], g.ny, true);
+          const int e2 = tile_offset(rvz, lo[2], g.nz, perz);
+          hit = (shx ? e0 <= hi[0] - lo[0] && e0 + SN - 1 >= 0
+                     : axis_reach<SN>(rvx, g.nx, true, lo[0], hi[0])) &&
+                (shy ? e1 <= hi[1] - lo[1] && e1 + SN - 1 >= 0
+                     : axis_reach<SN>(rvy, g.ny, true, lo[1], hi[1])) &&
+                (shz ? e2 <= hi[2] - lo[2] && e2 + SN - 1 >= 0
+                     : axis_reach<SN>(rvz, g.nz, perz, lo[2], hi[2]));
+        }
+        const unsigned m = __ballot_sync(full, hit);
+        if (hit) hk[nhit + __popc(m & ((1u << lane) - 1u))] = kk[r];
+        nhit += __popc(m);
+      }
+      __syncwarp();
+      for (int hb = 0; hb < nhit; hb += 32) {
+        const int nh = min(32, nhit - hb);
+        if (lane < nh) reduce_record<ST, C>(stage[lane], g, a, hk[hb + lane], lo);
+        __syncwarp();
+        for (int src = 0; src < nh; ++src) sum.add(stage[src], cxl, cyl, czl);
+        __syncwarp();
+      }
+    }
+  }
+  if (in0) store_force(F, cell0, sum.a[0][0], sum.a[1][0], sum.a[2][0]);
+  if (in1) store_force(F, cell1, sum.a[0][1], sum.a[1][1], sum.a[2][1]);
+  if (lane == 0) {
+    a.flag[t.x] = 1;
+    // the marks are consumed here, or by the pass over all tiles (spread_flags)
+    if (a.accumulate) a.mark[t.x] = 0u;
+  }
+}
+
+// A field that is not added to: the flags of the tiles no stencil reaches are
+// cleared, and the marks consumed (a live tile's flag is set by the warp that
+// spreads it: only the other flags are written).  Four tiles per thread and
+// access (marks and flags start 256-byte aligned), the remainder one by one.
+__device__ __forceinline__ void spread_flags(const Geom& g, const SpreadArgs& a, int bid, int nblk) {
+  const int ntiles = g.ntx * g.nty * g.ntz;
+  const long long gt = (long long)bid * blockDim.x + threadIdx.x;
+  const long long nthreads = (long long)nblk * blockDim.x;
+  const long long n4 = ntiles / 4;
+  uint4* mark4 = reinterpret_cast<uint4*>(a.mark);
+  uchar4* flag4 = reinterpret_cast<uchar4*>(a.flag);
+  for (long long q = gt; q < n4; q += nthreads) {
+    const uint4 m = mark4[q];
+    if ((m.x | m.y | m.z | m.w) == 0u) {
+      flag4[q] = make_uchar4(0, 0, 0, 0);
+    } else {
+      mark4[q] = make_uint4(0u, 0u, 0u, 0u);
+      uint8_t* f = a.flag + 4 * q;
+      if (!m.x) f[0] = 0;
+      if (!m.y) f[1] = 0;
+      if (!m.z) f[2] = 0;
+      if (!m.w) f[3] = 0;
+    }
+  }
+  for (long long t = 4 * n4 + gt; t < ntiles; t += nthreads) {
+    if (a.mark[t] != 0u) a.mark[t] = 0u;
+    else a.flag[t] = 0;
+  }
+}
+
+// Trilinear spreading from the hit lists, one warp per live tile.  Lane l owns
+// the cells (l & 3, (l >> 2) & 3, l >> 4) and the same cell two planes up and
+// adds the tile's markers in slot order (no atomics).  A tile is a chain of
+// four dependent loads (list entry, hits, records, the field it adds to), so
+// the chain is pipelined over the warp's tiles: while tile j is summed, the
+// records of its next tile, the hits of the one after and the list entry of
+// the third are in flight.  The markers are ordered by counting the smaller
+// slots (independent shuffles) instead of a sort, and their records are 32
+// bytes.  Axes of a single tile (where both nodes of a stencil can meet the
+// tile apart) and lists that overflowed take the search.  Bound by issue and
+// latency together (about 320 instructions per tile, 24 warps per SM):
+// 100 000 beads in 256^3 (34 000 live tiles) 34 -> 29 us per launch, 12 500
+// beads in 128^3 14.3 -> 10.6 us; half a warp per tile, four cells per lane,
+// took 40 us (more instructions per tile, not fewer: both halves wait for the
+// longer list), and a tile order that spreads a cluster over the SMs 30 us.
+template <typename C>
+__device__ __forceinline__ void spread_list_body(const PartArgs& __restrict__ p,
+                                                 const SpreadArgs& __restrict__ a, int bid, int nblk) {
+  constexpr unsigned full = 0xffffffffu;
+  static_assert(SPREAD_HCAP == 32, "one list entry per lane");
+  __shared__ SpreadHit<C> shit[SPREAD_WARPS][SPREAD_HCAP];
+  __shared__ int shk[SPREAD_WARPS][32 * SPREAD_ROUNDS];
+  const Geom& g = p.g;
+  const int lane = threadIdx.x & 31, wid = threadIdx.x >> 5;
+  SpreadHit<C>* stage = shit[wid];
+  const TriRecT<C>* recs = static_cast<const TriRecT<C>*>(a.rec);
+  C* F = static_cast<C*>(a.F);
+  const int ntiles = g.ntx * g.nty * g.ntz;
+  const int cx = lane & 3, cy = (lane >> 2) & 3, cz = lane >> 4;
+  const int stride = nblk * SPREAD_WARPS;
+  const int j0 = bid * SPREAD_WARPS + wid;
+  // (the list has room for every tile: entries are loaded ahead of the count)
+  auto entry = [&](int q) { return q < ntiles ? a.live_tiles[q] : make_int4(0, 0, 0, 0); };
+  int4 lt = entry(j0), lt1 = entry(j0 + stride), lt2 = entry(j0 + 2 * stride);
+  const int nlive = *a.nlive;
+  if (bid == 0 && threadIdx.x == 0) *a.nlive_next = 0;    // the next gather's counter (idle now)
+  const bool lists = g.ntx > 1 && g.nty > 1 && (g.walls || g.ntz > 1);
+  // length of a tile's list (beyond SPREAD_HCAP: the tile takes the search),
+  // the lane's entry, and whether the tile's field values are added to
+  auto count_of = [&](int q, const int4& t) { return q < nlive ? (int)a.hcnt[t.x] : 0; };
+  auto key_of_lane = [&](int q, const int4& t) {      // (entries past the count are not tiles)
+    return q < nlive ? a.hits[(size_t)t.x * SPREAD_HCAP + lane] : 0u;
+  };
+  auto rec_of = [&](int count, uint32_t key) {
+    TriRecT<C> r;
+    r.base = 0ull;
+#pragma unroll
+    for (int d = 0; d < 3; ++d) r.t[d] = r.F[d] = C(0);
+    if (lane < count && count <= SPREAD_HCAP) r = recs[key];
+    return r;
+  };
+  auto carry_of = [&](int q, const int4& t) { return q < nlive && a.accumulate && a.flag[t.x] != 0; };
+  bool overflow = false;
+  if (lists) {
+    int hc = count_of(j0, lt), hc1 = count_of(j0 + stride, lt1);
+    uint32_t key = key_of_lane(j0, lt), key1 = key_of_lane(j0 + stride, lt1);
+    bool carry = carry_of(j0, lt), carry1 = carry_of(j0 + stride, lt1);
+    TriRecT<C> rec = rec_of(hc, key);
+    for (int j = j0; j < nlive; j += stride) {
+      const int lo[3] = {lt.y * TILE, lt.z * TILE, lt.w * TILE};
+      const bool in0 = lo[0] + cx < g.nx && lo[1] + cy < g.ny && lo[2] + cz < g.nz;
+      const bool in1 = in0 && lo[2] + cz + 2 < g.nz;
+      const long long cell = (lo[2] + cz) * g.plane + (long long)(lo[1] + cy) * g.pitch + lo[0] + cx;
+      // the tile's field values, needed after its markers are staged, and
+      // the loads of the warp's next tiles
+      TileSum<C> sum;
+      sum.zero();
+      if (carry) {
+        if (in0) load_force(F, cell, sum.a[0][0], sum.a[1][0], sum.a[2][0]);
+        if (in1) load_force(F, cell + 2 * g.plane, sum.a[0][1], sum.a[1][1], sum.a[2][1]);
+      }
+      const TriRecT<C> rec1 = rec_of(hc1, key1);
+      const int hc2 = count_of(j + 2 * stride, lt2);
+      const uint32_t key2 = key_of_lane(j + 2 * stride, lt2);
+      const bool carry2 = carry_of(j + 2 * stride, lt2);
+      const int4 lt3 = entry(j + 3 * stride);
+      if (hc <= SPREAD_HCAP) {
+        // the marker's place: the number of smaller slots in the list
+        int rank = 0;
+#pragma unroll 4
+        for (int q = 0; q < hc; ++q) rank += __shfl_sync(full, key, q) < key ? 1 : 0;
+        if (lane < hc) {
+          SpreadHit<C>& h = stage[rank];
+          // the lower node's cell in the tile: 0 .. 3, or else the node lies
+          // one cell before the tile (a marker of the list reaches it)
+          const uint32_t b0 = (uint32_t)rec.base, b1 = (uint32_t)(rec.base >> 32);
+          const int b[3] = {(int)(b0 & 0x1FFFFFu), (int)(__funnelshift_r(b0, b1, 22) & 0x1FFFFFu),
+                            (int)b1 >> 11};
+#pragma unroll
+          for (int d = 0; d < 3; ++d) {
+            const int off = b[d] - lo[d];
+            const int e = (unsigned)off < (unsigned)TILE ? off : -1;
+            const C t0 = C(1) - rec.t[d], t1 = rec.t[d];
+            C w[TILE];
+#pragma unroll
+            for (int q = 0; q < TILE; ++q) w[q] = e == q ? t0 : (e == q - 1 ? t1 : C(0));
+            if (d == 0) put4(h.wx, w[0], w[1], w[2], w[3]);
+            else if (d == 1) put4(h.wy, w[0], w[1], w[2], w[3]);
+            else put4(h.wz, w[0], w[2], w[1], w[3]);
+          }
+          if constexpr (sizeof(C) == 4) {
+            put4(h.F, rec.F[0], rec.F[0], rec.F[1], rec.F[1]);
+            h.F[4] = rec.F[2];
+            h.F[5] = rec.F[2];
+          } else {
+            put4(h.F, rec.F[0], rec.F[1], rec.F[2], C(0));
+          }
+        }
+        __syncwarp();
+        for (int q = 0; q < hc; ++q) sum.add(stage[q], cx, cy, cz);
+        if (in0) store_force(F, cell, sum.a[0][0], sum.a[1][0], sum.a[2][0]);
+        if (in1) store_force(F, cell + 2 * g.plane, sum.a[0][1], sum.a[1][1], sum.a[2][1]);
+        if (lane == 0) {
+          a.flag[lt.x] = 1;
+          a.hcnt[lt.x] = 0u;                       // empty for the next gather
+          // the marks are consumed here, or by the pass over all tiles below
+          if (a.accumulate) a.mark[lt.x] = 0u;
+        }
+        __syncwarp();
+      } else {
+        overflow = true;
+      }
+      lt = lt1; lt1 = lt2; lt2 = lt3;
+      hc = hc1; hc1 = hc2;
+      key = key1; key1 = key2;
+      carry = carry1; carry1 = carry2;
+      rec = rec1;
+    }
+  }
+  // the tiles that take the search, in a loop of their own (its registers do
+  // not add to the list path's)
+  if (overflow || !lists)
+    for (int j = j0; j < nlive; j += stride) {
+      const int4 t = entry(j);
+      if (lists && a.hcnt[t.x] <= (uint32_t)SPREAD_HCAP) continue;
+      __syncwarp();
+      if (lane == 0) a.hcnt[t.x] = 0u;
+      spread_search_tile<0, C>(g, a, t, stage, shk[wid]);
+    }
+  if (!a.accumulate) spread_flags(g, a, bid, nblk);
+}
+
+// Spreading over the live tiles of one box (block bid of its nblk blocks),
+// taken from the list the gather built, a warp each: trilinear tiles from their
+// hit lists, the others by the search.
+template <int ST, typename C>
+__device__ __forceinline__ void spread_body(const PartArgs& __restrict__ p,
+                                            const SpreadArgs& __restrict__ a, int bid, int nblk) {
+  static_assert(TILE == 4 && TILE_CELLS == 64, "cells per lane");
+  if constexpr (ST == 0) {
+    spread_list_body<C>(p, a, bid, nblk);
+  } else {
+    __shared__ SpreadHit<C> shit[SPREAD_WARPS][32];
+    __shared__ int shk[SPREAD_WARPS][32 * SPREAD_ROUNDS];   // hits of a candidate group, in order
+    const Geom& g = p.g;
+    const int wid = threadIdx.x >> 5;
+    const int ntiles = g.ntx * g.nty * g.ntz;
+    const int stride = nblk * SPREAD_WARPS;
+    int j = bid * SPREAD_WARPS + wid;
+    auto entry = [&](int q) { return q < ntiles ? a.live_tiles[q] : make_int4(0, 0, 0, 0); };
+    int4 lt = entry(j);
+    const int nlive = *a.nlive;
+    if (bid == 0 && threadIdx.x == 0) *a.nlive_next = 0;    // the next gather's counter (idle now)
+    for (; j < nlive; j += stride) {
+      const int4 lt1 = entry(j + stride);
+      spread_search_tile<ST, C>(g, a, lt, shit[wid], shk[wid]);
+      lt = lt1;
+    }
+    if (!a.accumulate) spread_flags(g, a, bid, nblk);
+  }
+}
+
+// resident blocks per SM the spreading is compiled for: 80 registers without
+// spills.  At four blocks (64 registers) the spilled values cost more than the
+// warps gain: bead chains 256^3 888 against 892 us per step, 12 500 beads in
+// 128^3 285 against 298 us, rigid spheres (four-point) 584 against 606 us.
+constexpr int SPREAD_RESIDENT = 3;
+
+template <int ST, typename C>
+__global__ void __launch_bounds__(SPREAD_THREADS, SPREAD_RESIDENT)
 spread_kernel(const PartArgs p, const SpreadArgs a) {
   spread_body<ST, C>(p, a, blockIdx.x, gridDim.x);
 }

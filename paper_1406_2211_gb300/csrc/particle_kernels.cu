@@ -282,6 +282,18 @@ void neighbour_tiles(const Geom& g, int maxnt, int* table) {
   }
 }
 
+// blocks that give the spreading about one live tile per warp (a marker's
+// stencil reaches about 2 tiles (trilinear), 4 (three-point) or 8
+// (four-point), 8 warps a block), and its pass over the tiles' flags about
+// one access per thread
+long long spread_blocks(const PartArgs& p) {
+  const int per = p.stencil == 0 ? 2 : (p.stencil == 2 ? 4 : 8);
+  const long long tiles = (p.M * per + 7) / 8;
+  const long long flags = ((long long)p.g.ntx * p.g.nty * p.g.ntz + 4 * SPREAD_THREADS - 1) /
+                          (4 * SPREAD_THREADS);
+  return tiles > flags ? (tiles < 1 ? 1 : tiles) : flags;
+}
+
 template <int ST, typename C>
 static void spread_launch(const PartArgs& p, const SpreadArgs& a, cudaStream_t s) {
   // a persistent grid: as many blocks as fit on the device at once
@@ -293,7 +305,8 @@ static void spread_launch(const PartArgs& p, const SpreadArgs& a, cudaStream_t s
     cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per, spread_kernel<ST, C>, SPREAD_THREADS, 0);
     grids[dev] = sms * (per > 0 ? per : 1);
   }
-  spread_kernel<ST, C><<<grids[dev], SPREAD_THREADS, 0, s>>>(p, a);
+  const long long need = spread_blocks(p);
+  spread_kernel<ST, C><<<(unsigned)(need < grids[dev] ? need : grids[dev]), SPREAD_THREADS, 0, s>>>(p, a);
 }
 
 template <typename C>
