@@ -498,6 +498,13 @@ struct Plan {
         emit(OP_SMALL_SORT, e);
         ++n;
       }
+    } else if (b->M <= SORT_CLUSTER_MAX) {
+      launch_sort_cluster(b->M, kb, b->uptr(b->L.off_key[1]), b->uptr(b->L.off_idx[1]),
+                          b->uptr(b->L.off_key[0]), b->uptr(b->L.off_idx[0]),
+                          b->uptr(b->L.off_key[1]), b->uptr(b->L.off_idx[1]), b->L.ntiles,
+                          b->iptr(b->L.off_tb), b->iptr(b->L.off_te), b->uptr(b->L.off_home), need,
+                          changed_flag(), mcount, s);
+      ++n;
     } else {
       launch_sort(b->M, kb, b->uptr(b->L.off_key[1]), b->uptr(b->L.off_idx[1]),
                   b->uptr(b->L.off_key[0]), b->uptr(b->L.off_idx[0]), b->uptr(b->L.off_key[1]),

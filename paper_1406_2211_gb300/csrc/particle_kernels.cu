@@ -112,6 +112,53 @@ void launch_bins(int ntiles, long long M, const uint32_t* keys, const uint32_t* 
 
 long long small_sort_max() { return SMALL_SORT_MAX; }
 
+// blocks of the sort's cluster on the current device: 16 where the device can
+// hold such a cluster, else 8 (the portable size)
+static int sort_cluster_blocks() {
+  static int blocks[MAX_DEVICES] = {0};
+  const int dev = device_slot(nullptr);
+  if (blocks[dev] == 0) {
+    int n = 0;
+    cudaLaunchConfig_t cfg = {};
+    cudaLaunchAttribute at[1];
+    at[0].id = cudaLaunchAttributeClusterDimension;
+    at[0].val.clusterDim = {16, 1, 1};
+    cfg.gridDim = dim3(16);
+    cfg.blockDim = dim3(SORT_CLUSTER_THREADS);
+    cfg.attrs = at;
+    cfg.numAttrs = 1;
+    if (cudaFuncSetAttribute(sort_cluster_kernel, cudaFuncAttributeNonPortableClusterSizeAllowed, 1) !=
+            cudaSuccess ||
+        cudaOccupancyMaxActiveClusters(&n, sort_cluster_kernel, &cfg) != cudaSuccess) {
+      cudaGetLastError();
+      n = 0;
+    }
+    blocks[dev] = n > 0 ? 16 : 8;
+  }
+  return blocks[dev];
+}
+
+void launch_sort_cluster(long long M, int key_bits, const uint32_t* kin, const uint32_t* vin,
+                         uint32_t* ka, uint32_t* va, uint32_t* kb, uint32_t* vb, int ntiles, int* tb,
+                         int* te, uint32_t* home, const int* need, int* changed, int* brick_count,
+                         cudaStream_t s) {
+  if (M <= 0) return;
+  const int passes = sort_passes(key_bits);
+  const int width = (key_bits + passes - 1) / passes;
+  const int nb = sort_cluster_blocks();
+  cudaLaunchConfig_t cfg = {};
+  cudaLaunchAttribute at[1];
+  at[0].id = cudaLaunchAttributeClusterDimension;
+  at[0].val.clusterDim = {(unsigned)nb, 1, 1};
+  cfg.gridDim = dim3((unsigned)nb);
+  cfg.blockDim = dim3(SORT_CLUSTER_THREADS);
+  cfg.stream = s;
+  cfg.attrs = at;
+  cfg.numAttrs = 1;
+  cudaLaunchKernelEx(&cfg, sort_cluster_kernel, M, passes, width, kin, vin, ka, va, kb, vb, ntiles, tb,
+                     te, home, need, changed, brick_count);
+}
+
 void launch_small_sort_bins(long long M, int key_bits, const uint32_t* kin, const uint32_t* vin,
                             uint32_t* ka, uint32_t* va, int ntiles, int* tb, int* te,
                             uint32_t* home, const int* need, int* changed, int* brick_count,

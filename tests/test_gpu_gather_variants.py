@@ -23,7 +23,7 @@ def _resident():
     return 96 * torch.cuda.get_device_properties(0).multi_processor_count
 
 
-@pytest.mark.parametrize("count", [1, 5, "resident", "resident+1"])
+@pytest.mark.parametrize("count", [1, 5, 8193, "resident", "resident+1"])
 @pytest.mark.parametrize("split,n", [("base", 1), ("inside", 2)])
 @pytest.mark.parametrize("walls", [False, True])
 def test_trilinear_variants_match_oracle(count, split, n, walls):
