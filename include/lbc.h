@@ -269,8 +269,8 @@ lbc_status lbc_box_check(lbc_box* box, void* stream);
  *                  step) >= half the lattice's cells, M = max_particles.
  *  LBC_OPT_GATHER_LANES  lanes per marker in the interpolations of the
  *                  4- and 3-point stencils (without the per-marker node
- *                  cache of LBC_SPLIT_INSIDE): 1, 4 (each lane sums the
- *                  stencil rows ky = lane (mod 4), then the four parts are
+ *                  cache of LBC_SPLIT_INSIDE): 1, 4 (lane q sums the
+ *                  nodes kx = q of every stencil row, then the four parts are
  *                  added in a fixed order), or 0 = automatic (4 while the
  *                  markers are too few to fill the GPU one lane each).  The
  *                  two differ only in the order of the floating-point sum.

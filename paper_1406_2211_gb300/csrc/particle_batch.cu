@@ -14,7 +14,7 @@
 namespace lbc {
 
 int gather_variant(const PartArgs& p, const GatherArgs& a);
-int gather_lanes(int var);
+int gather_lanes(const PartArgs& p, int var);
 
 namespace {
 
@@ -94,12 +94,12 @@ small_sort_batch_kernel(const PartEntry* __restrict__ tab, int n) {
 
 template <typename S, bool WALLS, int ST, int VAR>
 __global__ void __launch_bounds__(GATHER_THREADS,
-                                  (VAR == GV_LIGHT || VAR == GV_CACHED || VAR == GV_OCT) ? 6 : 4)
+                                  gather_resident<ST, VAR, float>())
 gather_batch_kernel(const PartEntry* __restrict__ tab, int n) {
   __shared__ SharedEntry<HEAD + U_GM> se;
   const PartEntry& e = stage<U_GM>(tab, n, se);
   const long long gid = (blockIdx.x - e.block0) * (long long)blockDim.x + threadIdx.x;
-  if constexpr (VAR == GV_OCT) gather_oct_body<S, WALLS>(e.p, e.u.gm.g, gid);
+  if constexpr (VAR == GV_GROUP) gather_group_body<S, WALLS, ST>(e.p, e.u.gm.g, gid);
   else gather_body<S, WALLS, ST, VAR>(e.p, e.u.gm.g, gid);
 }
 
@@ -140,7 +140,7 @@ void gather_batch_st(int ST, unsigned grid, const PartEntry* tab, int n, cudaStr
 
 template <typename S, bool WALLS>
 void gather_batch_w(int ST, int var, unsigned grid, const PartEntry* tab, int n, cudaStream_t s) {
-  if (var == GV_OCT) gather_batch_kernel<S, WALLS, 0, GV_OCT><<<grid, GATHER_THREADS, 0, s>>>(tab, n);
+  if (var == GV_GROUP) gather_batch_st<S, WALLS, GV_GROUP>(ST, grid, tab, n, s);
   else if (var == GV_CACHED) gather_batch_st<S, WALLS, GV_CACHED>(ST, grid, tab, n, s);
   else if (var == GV_LIGHT) gather_batch_st<S, WALLS, GV_LIGHT>(ST, grid, tab, n, s);
   else gather_batch_st<S, WALLS, GV_FULL>(ST, grid, tab, n, s);
@@ -172,7 +172,6 @@ long long part_op_key(int kind, const PartEntry& e) {
     case OP_GATHER: {
       if (!c32) return -1;
       const int var = gather_variant(e.p, e.u.gm.g);
-      if (var == GV_QUAD) return -1;
       return (((long long)kind * 8 + st) * 2 + e.p.g.walls) * 64 + e.p.stencil * 8 + var;
     }
     case OP_SPREAD:
@@ -192,7 +191,7 @@ int part_op_blocks(int kind, const PartEntry& e) {
     case OP_DRIFT:
       return (int)((M + GATHER_THREADS - 1) / GATHER_THREADS);
     case OP_GATHER:
-      return (int)((gather_lanes(gather_variant(e.p, e.u.gm.g)) * M + GATHER_THREADS - 1) /
+      return (int)((gather_lanes(e.p, gather_variant(e.p, e.u.gm.g)) * M + GATHER_THREADS - 1) /
                    GATHER_THREADS);
     case OP_SMALL_SORT:
       return 1;

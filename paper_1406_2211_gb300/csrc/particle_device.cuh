@@ -1324,21 +1324,13 @@ __device__ __forceinline__ bool gather_field(const GatherArgs& a, const Geom& g,
 //              two nodes at a time (or reads the node-moment field);
 //   GV_LIGHT   the same for launches that read the node-moment field (fewer
 //              registers, more markers in flight);
-//   GV_QUAD    (4- and 3-point stencils, no node cache, no fused drift; by
-//              default only for fewer markers than the one-lane variants
-//              keep resident at once) four lanes per marker, lane q taking
-//              the stencil rows ky = q (mod 4) of every plane, their parts
-//              summed with a fixed butterfly: four times the loads in flight
-//              for the same markers.  Lane 0 of a group does the marker's
-//              update and writes its record; the tile claims are shared out
-//              by plane;
 //   GV_CACHED  one lane per marker with the node cache: markers whose cache
 //              entry does not hold are refilled by the whole warp first
 //              (refill_cache), then every lane reads its nodes from the
 //              cache with all loads in flight;
-//   GV_OCT     (trilinear) eight lanes per marker, one per node
-//              (gather_oct_body).
-constexpr int GV_FULL = 0, GV_LIGHT = 1, GV_QUAD = 2, GV_CACHED = 3, GV_OCT = 4;
+//   GV_GROUP   a group of lanes per marker (gather_group_body): eight for the
+//              trilinear stencil, one per node, four for the others.
+constexpr int GV_FULL = 0, GV_LIGHT = 1, GV_CACHED = 2, GV_GROUP = 3;
 
 // Coupling force F^h of N components from the slip dv = v - u(X), the
 // intrinsic force Fi and the random force zeta (compute type)
@@ -1521,6 +1513,66 @@ __device__ __forceinline__ int claim_slots(int* nlive, int nclaim, unsigned am, 
   return __shfl_sync(am, base, nact - 1) + incl - nclaim;
 }
 
+// The tile claims of a 4- or 3-point stencil: loops over the distinct tiles per
+// axis instead of the SN^3 node combinations: per axis the distinct tiles of
+// the nodes with non-zero weight, in node order (at most three: a partial last
+// tile and the periodic wrap), their combinations shared out over the
+// marker's GL lanes.
+template <int SN, int GL, typename C>
+__device__ __forceinline__ void claim_wide(const GatherArgs& a, const Geom& g, const int (&b)[3],
+                                           const C (&w)[3][4], int sub, bool valid, unsigned am, int nact) {
+  const int n3[3] = {g.nx, g.ny, g.nz};
+  const bool per[3] = {true, true, !g.walls};
+  int tl[3][3], ntl[3];
+  uint32_t claimed = 0u;               // bit of the tile combination cid
+  int nclaim = 0;
+#pragma unroll
+  for (int c = 0; c < 3; ++c) {
+    ntl[c] = 0;
+    tl[c][0] = tl[c][1] = tl[c][2] = -1;
+#pragma unroll
+    for (int q = 0; q < SN; ++q) {
+      if (w[c][q] == C(0)) continue;
+      int node = b[c] + q;
+      if (per[c]) node = wrap_int(node, n3[c]);
+      if (node < 0 || node >= n3[c]) continue;
+      const int t = node >> TILE_SHIFT;
+      if (t == tl[c][0] || t == tl[c][1] || t == tl[c][2]) continue;
+      if (ntl[c] == 0) tl[c][0] = t;
+      else if (ntl[c] == 1) tl[c][1] = t;
+      else tl[c][2] = t;
+      ++ntl[c];
+    }
+  }
+  // claim the tiles the stencil reaches: the combinations of the axes'
+  // tiles, shared out over the marker's lanes
+  int cid = 0;
+  for (int iz = 0; iz < ntl[2]; ++iz)
+    for (int iy = 0; iy < ntl[1]; ++iy)
+      for (int ix = 0; ix < ntl[0]; ++ix, ++cid) {
+        if (cid % GL != sub || !valid) continue;
+        const int tx = pick(tl[0], ix), ty = pick(tl[1], iy), tz = pick(tl[2], iz);
+        // most tiles are claimed already: an L2 read (marks only go
+        // from 0 to 1 during the gather) spares their atomic
+        uint32_t* m = a.mark + (tz * g.nty + ty) * g.ntx + tx;
+        if (__ldcg(m) == 0u && atomicExch(m, 1u) == 0u) {
+          claimed |= 1u << cid;
+          ++nclaim;
+        }
+      }
+  int base = claim_slots(a.nlive, nclaim, am, nact);
+  if (claimed != 0u) {
+    int cid2 = 0;
+    for (int iz = 0; iz < ntl[2]; ++iz)
+      for (int iy = 0; iy < ntl[1]; ++iy)
+        for (int ix = 0; ix < ntl[0]; ++ix, ++cid2)
+          if (claimed & (1u << cid2)) {
+            const int tx = pick(tl[0], ix), ty = pick(tl[1], iy), tz = pick(tl[2], iz);
+            a.live_tiles[base++] = make_int4((tz * g.nty + ty) * g.ntx + tx, tx, ty, tz);
+          }
+  }
+}
+
 // the body of the gather for thread gid of one box's launch (whole warps of
 // one box: gid - lane is a multiple of 32)
 template <typename S, bool WALLS, int ST, int VAR>
@@ -1528,7 +1580,7 @@ __device__ __forceinline__ void gather_body(const PartArgs& __restrict__ p,
                                             const GatherArgs& __restrict__ a, long long gid) {
   using C = typename Store<S>::C;
   constexpr int SN = nodes_1d<ST>();
-  constexpr int GL = VAR == GV_QUAD ? 4 : 1;       // lanes per marker
+  constexpr int GL = 1;
   constexpr bool CACHED = VAR == GV_CACHED;
   const Geom& g = p.g;
   const long long M = p.M;
@@ -1799,64 +1851,78 @@ __device__ __forceinline__ void gather_body(const PartArgs& __restrict__ p,
           a.live_tiles[base++] = make_int4((tz * g.nty + ty) * g.ntx + tx, tx, ty, tz);
         }
     } else {
-      // 4- and 3-point stencils: loops over the distinct tiles per axis
-      // instead of the SN^3 node combinations: per axis the distinct tiles
-      // of the nodes with non-zero weight, in node order (at most three: a
-      // partial last tile and the periodic wrap)
-      int tl[3][3], ntl[3];
-      uint32_t claimed = 0u;               // bit of the tile combination cid
-      int nclaim = 0;
-#pragma unroll
-      for (int c = 0; c < 3; ++c) {
-        ntl[c] = 0;
-        tl[c][0] = tl[c][1] = tl[c][2] = -1;
-#pragma unroll
-        for (int q = 0; q < SN; ++q) {
-          if (w[c][q] == C(0)) continue;
-          int node = b[c] + q;
-          if (per[c]) node = wrap_int(node, n3[c]);
-          if (node < 0 || node >= n3[c]) continue;
-          const int t = node >> TILE_SHIFT;
-          if (t == tl[c][0] || t == tl[c][1] || t == tl[c][2]) continue;
-          if (ntl[c] == 0) tl[c][0] = t;
-          else if (ntl[c] == 1) tl[c][1] = t;
-          else tl[c][2] = t;
-          ++ntl[c];
-        }
-      }
-      // claim the tiles the stencil reaches: the combinations of the axes'
-      // tiles, shared out over the marker's lanes
-      int cid = 0;
-      for (int iz = 0; iz < ntl[2]; ++iz)
-        for (int iy = 0; iy < ntl[1]; ++iy)
-          for (int ix = 0; ix < ntl[0]; ++ix, ++cid) {
-            if (cid % GL != sub || !valid) continue;
-            const int tx = pick(tl[0], ix), ty = pick(tl[1], iy), tz = pick(tl[2], iz);
-            // most tiles are claimed already: an L2 read (marks only go
-            // from 0 to 1 during the gather) spares their atomic
-            uint32_t* m = a.mark + (tz * g.nty + ty) * g.ntx + tx;
-            if (__ldcg(m) == 0u && atomicExch(m, 1u) == 0u) {
-              claimed |= 1u << cid;
-              ++nclaim;
-            }
-          }
-      int base = claim_slots(a.nlive, nclaim, am, nact);
-      if (claimed != 0u) {
-        int cid2 = 0;
-        for (int iz = 0; iz < ntl[2]; ++iz)
-          for (int iy = 0; iy < ntl[1]; ++iy)
-            for (int ix = 0; ix < ntl[0]; ++ix, ++cid2)
-              if (claimed & (1u << cid2)) {
-                const int tx = pick(tl[0], ix), ty = pick(tl[1], iy), tz = pick(tl[2], iz);
-                a.live_tiles[base++] = make_int4((tz * g.nty + ty) * g.ntx + tx, tx, ty, tz);
-              }
-      }
+      claim_wide<SN, GL, C>(a, g, b, w, sub, valid, am, nact);
     }
   }
 }
 
-// The trilinear interpolation with eight lanes per marker (every mode; with
-// or without the node cache and the fused drift).  Lane q owns node
+// One lane's column of a 4- or 3-point stencil (x fixed; rows ys, planes zs)
+// from the node-moment field, two planes of rows with their loads in flight
+// together.  The rows lie in the tiles of the first and the last row (else, or
+// where a tile is not ready, false is returned and own is to be redone node by
+// node), so the ready bytes and force flags are loaded for two tiles a plane.
+// HAS: the force field F1 is added.
+template <int SN, bool HAS, typename C>
+__device__ __forceinline__ bool wide_column(const GatherArgs& __restrict__ a, const Geom& g, int x,
+                                            const int (&ys)[SN], const int (&zs)[SN], C wx,
+                                            const C (&w)[3][4], const C (&cgg)[3], C (&own)[3]) {
+  const C* mom = static_cast<const C*>(a.mom);
+  const C* F1 = static_cast<const C*>(a.F1);
+  const C c1 = rv<C>(a.c1);
+  const int tx = x >> TILE_SHIFT, ty0 = ys[0] >> TILE_SHIFT, ty1 = ys[SN - 1] >> TILE_SHIFT;
+  bool ok = true;
+#pragma unroll
+  for (int q = 1; q < SN - 1; ++q) ok &= (ys[q] >> TILE_SHIFT) == ty0 || (ys[q] >> TILE_SHIFT) == ty1;
+  if (!ok) return false;
+#pragma unroll 1
+  for (int k0 = 0; k0 < SN; k0 += 2) {
+    C j[2][SN][3], inv[2][SN], f[2][SN][3];
+    bool on[2][2], in[2];
+#pragma unroll
+    for (int h = 0; h < 2; ++h) {
+      const int z = k0 + h < SN ? pick(zs, k0 + h) : -1;
+      in[h] = z >= 0;                                  // a plane of the stencil, not beyond a wall
+      on[h][0] = on[h][1] = false;
+      if (!in[h]) continue;
+      const int t0 = ((z >> TILE_SHIFT) * g.nty + ty0) * g.ntx + tx, t1 = t0 + (ty1 - ty0) * g.ntx;
+      ok &= a.mready[t0] != 0 && a.mready[t1] != 0;
+      if (HAS) {
+        on[h][0] = a.flag1[t0] != 0;
+        on[h][1] = a.flag1[t1] != 0;
+      }
+#pragma unroll
+      for (int ky = 0; ky < SN; ++ky) {
+        const long long cell = z * g.plane + (long long)ys[ky] * g.pitch + x;
+        cache_load(mom + 4 * cell, j[h][ky], inv[h][ky]);
+        if (HAS) load_force(F1, cell, f[h][ky][0], f[h][ky][1], f[h][ky][2]);
+      }
+    }
+#pragma unroll
+    for (int h = 0; h < 2; ++h) {
+      if (!in[h]) continue;
+      const C wxz = wx * pick(w[2], k0 + h);
+#pragma unroll
+      for (int ky = 0; ky < SN; ++ky) {
+        const bool o = HAS && ((ys[ky] >> TILE_SHIFT) == ty0 ? on[h][0] : on[h][1]);
+        const C wt = wxz * w[1][ky];
+#pragma unroll
+        for (int c = 0; c < 3; ++c) {
+          C v = j[h][ky][c];
+          if (HAS) v = o ? v + c1 * f[h][ky][c] : v;
+          v += cgg[c];
+          own[c] += wt * (v * inv[h][ky]);
+        }
+      }
+    }
+  }
+  return ok;
+}
+
+// The interpolation with a group of lanes per marker, all of its lanes taking
+// part in every stage.
+//
+// Trilinear: eight lanes per marker (every mode; with or without the node
+// cache and the fused drift).  Lane q owns node
 // (q & 1, (q >> 1) & 1, q >> 2): its cache entry, field entry or 19
 // populations are loaded side by side with the other nodes', the node
 // velocities are added in node order through shuffles (the same sum as with
@@ -1865,18 +1931,29 @@ __device__ __forceinline__ void gather_body(const PartArgs& __restrict__ p,
 // markers lasts as long as one marker's chain of dependent loads, which is
 // about one load per stage here (1000 markers, populations pulled: 34 us per
 // launch with one lane, whole step of the 64^3 box 66 -> 39 us).
-template <typename S, bool WALLS>
-__device__ __forceinline__ void gather_oct_body(const PartArgs& __restrict__ p,
+//
+// 4- and 3-point stencils (no node cache, no fused drift): four lanes per
+// marker, lane q owning the nodes kx = q of every row, so a row of the stencil
+// is one contiguous access of the group; the lanes' parts are summed with a
+// fixed butterfly.  What bounds the wide stencils is L1's tag lookups, one per
+// distinct line of a request: one lane per marker (or one row per lane) sends
+// 32 lines per load, a group per row about 11.
+// 41 088 shell markers in 192^3 42 -> 30 us per launch (a row per lane before),
+// shell step 387 -> 350 us, one shell in 48^3 58 -> 54 us.
+template <typename S, bool WALLS, int ST>
+__device__ __forceinline__ void gather_group_body(const PartArgs& __restrict__ p,
                                                 const GatherArgs& __restrict__ a, long long gid) {
   using C = typename Store<S>::C;
+  constexpr int SN = nodes_1d<ST>();
+  constexpr int GL = ST == 0 ? 8 : 4;
   const Geom& g = p.g;
   const long long M = p.M;
   const int lane = threadIdx.x & 31;
-  const long long k = gid >> 3;
-  const int sub = lane & 7, lead = lane & ~7;
+  const long long k = gid / GL;
+  const int sub = lane & (GL - 1), lead = lane & ~(GL - 1);
   if (k >= M) return;                  // whole groups leave together
   const long long wbase = gid - lane;
-  const int nact = 8 * M - wbase >= 32 ? 32 : (int)(8 * M - wbase);
+  const int nact = GL * M - wbase >= 32 ? 32 : (int)(GL * M - wbase);
   const unsigned am = nact == 32 ? 0xffffffffu : ((1u << nact) - 1u);
   const long long i = a.perm ? (long long)a.perm[k] : k;
   const int n3[3] = {g.nx, g.ny, g.nz};
@@ -1884,7 +1961,7 @@ __device__ __forceinline__ void gather_oct_body(const PartArgs& __restrict__ p,
   const int comp = sub < 3 ? sub : 2;             // the lane's component
   int4 cb = make_int4(0, 0, 0, 0);
   bool try_reuse = false;
-  if (a.cache == 2) {
+  if (ST == 0 && a.cache == 2) {
     cb = a.ncache_b[k];
     try_reuse = a.invalidate == nullptr || *a.invalidate == 0;
   }
@@ -1892,7 +1969,7 @@ __device__ __forceinline__ void gather_oct_body(const PartArgs& __restrict__ p,
   const bool at_aux = a.mode == GM_IBM_HALF || a.mode == GM_IBM_FINAL;
   double X[3], vc = 0.0, im = 0.0;
   C Fc = C(0);
-  if (a.fused) {
+  if (ST == 0 && a.fused) {
     double v[3];
     C F[3];
     im = a.inv_mass[i];
@@ -1923,13 +2000,14 @@ __device__ __forceinline__ void gather_oct_body(const PartArgs& __restrict__ p,
     if constexpr (sizeof(C) == 4) {
       float xh, xl;
       split_df(X[c], xh, xl);
-      stencil_1d_df<0>(xh, xl, b[c], w[c]);
+      stencil_1d_df<ST>(xh, xl, b[c], w[c]);
     } else {
-      stencil_1d<0, C>(X[c], b[c], w[c]);
+      stencil_1d<ST, C>(X[c], b[c], w[c]);
     }
   }
   C own[3] = {C(0), C(0), C(0)};
   if (a.mode != GM_IBM1) {
+    if constexpr (ST == 0) {
     const int x = wrap_int(b[0] + (sub & 1), g.nx), y = wrap_int(b[1] + ((sub >> 1) & 1), g.ny);
     int z = b[2] + (sub >> 2);
     if (!WALLS) z = wrap_int(z, g.nz);
@@ -1966,6 +2044,41 @@ __device__ __forceinline__ void gather_oct_body(const PartArgs& __restrict__ p,
         const C u = __shfl_sync(am, nv[c], lead + q);
         if (node_in) own[c] += wt * u;
       }
+    }
+    } else {
+    // lane q: the nodes kx = q of the rows, row by row
+    int ys[SN], zs[SN];
+#pragma unroll
+    for (int q = 0; q < SN; ++q) {
+      ys[q] = wrap_int(b[1] + q, g.ny);
+      const int zz = b[2] + q;
+      zs[q] = WALLS ? ((zz < 0 || zz >= g.nz) ? -1 : zz) : wrap_int(zz, g.nz);
+    }
+    const int x = wrap_int(b[0] + sub, g.nx);
+    const C wx = pick(w[0], sub);
+    const C cgg[3] = {rv<C>(a.cgg[0]), rv<C>(a.cgg[1]), rv<C>(a.cgg[2])};
+    if (sub < SN) {
+      bool done = false;
+      if (a.mom != nullptr && a.F2 == nullptr)
+        done = a.F1 != nullptr ? wide_column<SN, true, C>(a, g, x, ys, zs, wx, w, cgg, own)
+                               : wide_column<SN, false, C>(a, g, x, ys, zs, wx, w, cgg, own);
+      if (!done) {
+        own[0] = own[1] = own[2] = C(0);
+#pragma unroll 1
+        for (int kz = 0; kz < SN; ++kz) {
+          const int z = pick(zs, kz);
+          if (WALLS && z < 0) continue;
+          const C wxz = wx * pick(w[2], kz);
+#pragma unroll 1
+          for (int ky = 0; ky < SN; ++ky)
+            gather_node<S, WALLS>(a, g, x, pick(ys, ky), z, wxz * pick(w[1], ky), cgg, own);
+        }
+      }
+    }
+#pragma unroll
+    for (int off = 1; off < GL; off <<= 1)
+#pragma unroll
+      for (int c = 0; c < 3; ++c) own[c] += __shfl_xor_sync(am, own[c], off);
     }
   }
   // ---- the marker's update, one component per lane
@@ -2015,9 +2128,10 @@ __device__ __forceinline__ void gather_oct_body(const PartArgs& __restrict__ p,
     const C Frec[3] = {__shfl_sync(am, frec, lead), __shfl_sync(am, frec, lead + 1),
                        __shfl_sync(am, frec, lead + 2)};
     if (sub == 0) {
-      write_record<0>(a, g, k, b, w, Frec);
-      if (a.keys && !bins_hold<2>(g, home, b)) *a.status = 1;
+      write_record<ST>(a, g, k, b, w, Frec);
+      if (a.keys && !bins_hold<SN>(g, home, b)) *a.status = 1;
     }
+    if constexpr (ST == 0) {
     int tq[3][2];
 #pragma unroll
     for (int c = 0; c < 3; ++c) axis_tiles<2>(b[c], w[c], n3[c], per[c], tq[c]);
@@ -2036,16 +2150,25 @@ __device__ __forceinline__ void gather_oct_body(const PartArgs& __restrict__ p,
     if (lane == 0 && m != 0u) base = atomicAdd(a.nlive, __popc(m));
     base = __shfl_sync(am, base, 0);
     if (first) a.live_tiles[base + __popc(m & ((1u << lane) - 1u))] = make_int4(tile, tx, ty, tz);
+    } else {
+      claim_wide<SN, GL, C>(a, g, b, w, sub, true, am, nact);
+    }
   }
+}
+
+// resident blocks per SM a variant is compiled for
+template <int ST, int VAR, typename C>
+constexpr int gather_resident() {
+  if (VAR == GV_GROUP && ST != 0) return 4;       // two planes of loads in registers
+  return VAR != GV_FULL && sizeof(C) == 4 ? 6 : 4;
 }
 
 template <typename S, bool WALLS, int ST, int VAR>
 __global__ void __launch_bounds__(GATHER_THREADS,
-                                  ((VAR == GV_LIGHT || VAR == GV_CACHED || VAR == GV_OCT) &&
-                                   sizeof(typename Store<S>::C) == 4) ? 6 : 4)
+                                  gather_resident<ST, VAR, typename Store<S>::C>())
 gather_kernel(const PartArgs p, const GatherArgs a) {
   const long long gid = blockIdx.x * (long long)blockDim.x + threadIdx.x;
-  if constexpr (VAR == GV_OCT) gather_oct_body<S, WALLS>(p, a, gid);
+  if constexpr (VAR == GV_GROUP) gather_group_body<S, WALLS, ST>(p, a, gid);
   else gather_body<S, WALLS, ST, VAR>(p, a, gid);
 }
 

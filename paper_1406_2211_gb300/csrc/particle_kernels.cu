@@ -177,17 +177,18 @@ void launch_small_sort_bins(long long M, int key_bits, const uint32_t* kin, cons
                                                              brick_count);
 }
 
-// markers the one-lane variants keep resident at once (6 blocks of 128
-// threads per SM); below that the four-lane variant fills the GPU better
+// 4- and 3-point stencils: a group of four lanes per marker while the markers
+// are fewer than the one-lane variants keep resident at once (6 blocks of 128
+// threads per SM); beyond that the groups' repeated per-marker work and waves
+// of long chains cost more than the lines they save (200 000 sphere markers:
+// 549 us per step with one lane, 685 with four).
 static long long one_lane_wave() {
-  static long long w[MAX_DEVICES] = {0};
   int sms = 0;
-  const int dev = device_slot(&sms);
-  if (w[dev] == 0) w[dev] = (long long)sms * 6 * GATHER_THREADS;
-  return w[dev];
+  device_slot(&sms);
+  return (long long)sms * 6 * GATHER_THREADS;
 }
 
-// Trilinear: eight lanes per marker (GV_OCT) up to the markers whose lanes
+// Trilinear: eight lanes per marker (GV_GROUP) up to the markers whose lanes
 // are resident at once (6 blocks of 128 threads per SM, 96 markers per SM):
 // below that a launch lasts as long as one marker's chain, which the lanes
 // shorten; above it their repeated per-marker work fills the issue slots.
@@ -205,10 +206,10 @@ static long long oct_max() {
 // decides the order of the floating-point sums, so a batched launch uses the
 // same one)
 int gather_variant(const PartArgs& p, const GatherArgs& a) {
-  if (p.stencil == 0 && p.M <= oct_max()) return GV_OCT;
+  if (p.stencil == 0 && p.M <= oct_max()) return GV_GROUP;
   if (a.cache != 0) return GV_CACHED;
-  const bool quad_ok = p.stencil != 0 && !a.fused;
-  if (quad_ok && (a.lanes == 4 || (a.lanes == 0 && p.M < one_lane_wave()))) return GV_QUAD;
+  if (p.stencil != 0 && !a.fused && (a.lanes == 4 || (a.lanes == 0 && p.M < one_lane_wave())))
+    return GV_GROUP;
   // the lighter variant spills with the wall bounce-back of the pull, which
   // the field reads still need where a tile is not ready
   if (a.mom != nullptr && !p.g.walls) return GV_LIGHT;
@@ -216,13 +217,13 @@ int gather_variant(const PartArgs& p, const GatherArgs& a) {
 }
 
 // lanes per marker of a variant
-int gather_lanes(int var) { return var == GV_OCT ? 8 : (var == GV_QUAD ? 4 : 1); }
+int gather_lanes(const PartArgs& p, int var) { return var != GV_GROUP ? 1 : (p.stencil == 0 ? 8 : 4); }
 
 template <typename S, bool WALLS>
 static void gather_st(const PartArgs& p, const GatherArgs& a, cudaStream_t s) {
   const int var = gather_variant(p, a);
   const int bs = GATHER_THREADS;
-  const unsigned nb = (unsigned)((gather_lanes(var) * p.M + bs - 1) / bs);
+  const unsigned nb = (unsigned)((gather_lanes(p, var) * p.M + bs - 1) / bs);
 #define LBC_G(ST, V) gather_kernel<S, WALLS, ST, V><<<nb, bs, 0, s>>>(p, a)
 #define LBC_GS(V)                                       \
   do {                                                  \
@@ -231,10 +232,7 @@ static void gather_st(const PartArgs& p, const GatherArgs& a, cudaStream_t s) {
     else LBC_G(2, V);                                   \
   } while (0)
   switch (var) {
-    case GV_OCT: LBC_G(0, GV_OCT); break;
-    case GV_QUAD:
-      if (p.stencil == 1) LBC_G(1, GV_QUAD); else LBC_G(2, GV_QUAD);
-      break;
+    case GV_GROUP: LBC_GS(GV_GROUP); break;
     case GV_CACHED: LBC_GS(GV_CACHED); break;
     case GV_LIGHT: LBC_GS(GV_LIGHT); break;
     default: LBC_GS(GV_FULL); break;
