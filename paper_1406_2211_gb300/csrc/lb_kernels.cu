@@ -30,7 +30,7 @@ namespace lbc {
 // block = bx x by cells of one z plane (bx * by <= 256; the shape is the
 // tuning parameter, see lbc_box_autotune)
 template <typename S, int COLL, bool WALLS, bool FORCED, typename IX>
-__global__ void __launch_bounds__(256, 5)
+__global__ void __launch_bounds__(256, sizeof(typename Store<S>::C) == 8 ? 2 : 5)
 lb_step_kernel(const S* __restrict__ fin, S* __restrict__ fout, const LBArgs a) {
   const int x = blockIdx.x * blockDim.x + threadIdx.x;
   const int y = blockIdx.y * blockDim.y + threadIdx.y;
