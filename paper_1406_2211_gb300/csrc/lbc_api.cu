@@ -200,7 +200,7 @@ struct lbc_box {
   cudaGraphExec_t graph[2];   // two-step graphs, by starting parity of cur
   cudaGraph_t tgraph[2];      // their templates (node handles for updates)
   cudaStream_t graph_stream[2];
-  int graph_lv[2];            // lv at the capture
+  int graph_lv[2], graph_pc[2];   // lv and pc at the capture
   // LB-kernel timing: event pairs around every LB launch (see LBC_OPT_TIMING)
   int64_t timing_cap;         // pairs available (0 = off)
   int64_t timing_used;        // pairs recorded since the last reset
@@ -699,10 +699,12 @@ void enqueue_step(lbc_box* b, cudaStream_t s, int64_t* launches, int phase = 0,
     a.mode = GM_COUPLE; a.s = make_real(h); a.include_int = 1; a.rec_weight = make_real(1.0);
     P.fields(a, -1, 0.0, -1, 0.0, 0.0);
     P.noise(a, 0, h);
+    // r += h v follows the kick in the same kernel (nothing else reads the
+    // position before the step's end: the spreading has its records)
+    a.pos_next = a.pos; a.post_a = h; a.post_b = 0.0;
     P.gather(a);
     P.spread(ib, false);
     P.lb(nullptr, b->F(ib), 0.0, h, h);
-    P.drift(h, 0.0, 0.0, false, false);
     *launches += P.n;
     return;
   }
@@ -722,9 +724,10 @@ void enqueue_step(lbc_box* b, cudaStream_t s, int64_t* launches, int phase = 0,
     a.mode = GM_COUPLE; a.s = make_real(0.5 * h); a.include_int = 1; a.rec_weight = make_real(1.0);
     P.fields(a, -1, 0.0, -1, 0.0, 0.0);
     P.noise(a, 1, 0.5 * h);
+    // the closing half drift follows the kick in the same kernel
+    a.pos_next = a.pos; a.post_a = 0.5 * h; a.post_b = 0.0;
     P.gather(a);
     P.spread(ia, false);
-    P.drift(0.5 * h, 0.0, 0.0, false, false);
   } else if (split == LBC_SPLIT_INSIDE) {
     // Eq. [multistep]: n Verlet sub-steps with coupling on each side of LB.
     // Every sub-step is one kernel: the drift to its force point, the
@@ -882,7 +885,8 @@ lbc_status run_steps(lbc_box* b, int64_t nsteps, cudaStream_t s) {
   }
   if (nsteps <= 0) return LBC_OK;
   const int par = b->cur;
-  if (!b->graph[par] || b->graph_stream[par] != s || b->graph_lv[par] != b->lv) {
+  if (!b->graph[par] || b->graph_stream[par] != s || b->graph_lv[par] != b->lv ||
+      b->graph_pc[par] != b->pc) {
     if (b->graph[par]) {
       cudaGraphExecDestroy(b->graph[par]);
       b->graph[par] = nullptr;
@@ -937,6 +941,7 @@ lbc_status run_steps(lbc_box* b, int64_t nsteps, cudaStream_t s) {
     b->tgraph[par] = graph;
     b->graph_stream[par] = s;
     b->graph_lv[par] = lv0;
+    b->graph_pc[par] = pc0;
   }
   while (nsteps >= 2) {
     if (b->timing_cap > 0 && b->tnode[par][0]) {
