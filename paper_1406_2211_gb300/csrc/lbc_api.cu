@@ -1759,13 +1759,14 @@ extern "C" lbc_status lbc_box_autotune(lbc_box* b, void* stream, int32_t* block_
 }
 
 // ------------------------------------------------------------ batching
-// Members advance together: per batched step, the phase-1 part of every
-// member's step (particle work before its LB step) runs on the member's own
-// stream, the LB steps of all members run as one launch per group (storage,
-// collision variant, walls, forcing) over a box table, then the phase-2
-// parts run on the member streams again.  Two batched steps are captured as
-// one CUDA graph per step parity and replayed while the membership is
-// unchanged.
+// Members advance together, in one of two ways (batch_recordable):
+//  batched: the particle work before the LB steps of all members runs as one
+//    launch per operation, the LB steps as one launch per group (storage,
+//    collision variant, walls, forcing) over a box table, then the particle
+//    work after them again as one launch per operation;
+//  streams: every member's whole steps run on a stream of its own.
+// Two batched steps are captured as one CUDA graph per step parity and
+// replayed while the membership is unchanged.
 struct lbc_batch {
   struct Member {
     lbc_box* box;
@@ -1925,19 +1926,16 @@ void batch_reset_graphs(lbc_batch* B) {
 // particle operations in `phost`; they must be on the device before the
 // launches run: with copy = true they are copied on `main` here (eager
 // steps); during capture the caller copies them after the capture ends.
-// When every member's particle work can be recorded (batch_recordable), the
-// part of each member's step before its LB step and the part after it are
-// recorded and run as one launch per operation for all members (run_ops);
-// otherwise each member's parts run on the member's own stream.
+// The part of each member's step before its LB step and the part after it are
+// recorded and run as one launch per operation for all members (run_ops).
 lbc_status batch_step(lbc_batch* B, cudaStream_t main, int region, std::vector<BoxEntry>& host,
                       std::vector<PartEntry>& phost, bool copy, int64_t* launches) {
   const int n = (int)B->members.size();
   BoxEntry* dev = region_boxes(B, region);
   PartEntry* pdev = region_parts(B, region);
-  const bool rec = batch_recordable(B);
   phost.clear();
   int64_t l = 0;
-  if (rec) {
+  {
     std::vector<OpList> ops(n);
     for (int j = 0; j < n; ++j) {
       int64_t lj = 0;
@@ -1945,17 +1943,6 @@ lbc_status batch_step(lbc_batch* B, cudaStream_t main, int region, std::vector<B
     }
     lbc_status st = run_ops(B, main, ops, pdev, phost, copy, &l);
     if (st != LBC_OK) return st;
-  } else {
-    CK(cudaEventRecord(B->fork[0], main));
-    for (int j = 0; j < n; ++j) {
-      cudaStream_t sj = B->streams[j];
-      CK(cudaStreamWaitEvent(sj, B->fork[0], 0));
-      int64_t lj = 0;
-      enqueue_step(B->members[j].box, sj, &lj, 1);
-      l += lj;
-      CK(cudaEventRecord(B->events[j], sj));
-      CK(cudaStreamWaitEvent(main, B->events[j], 0));
-    }
   }
   // group the recorded LB steps; rows are numbered per group in table order
   struct Key {
@@ -2003,7 +1990,7 @@ lbc_status batch_step(lbc_batch* B, cudaStream_t main, int region, std::vector<B
                       main);
     ++l;
   }
-  if (rec) {
+  {
     std::vector<OpList> ops(n);
     for (int j = 0; j < n; ++j) {
       int64_t lj = 0;
@@ -2011,19 +1998,38 @@ lbc_status batch_step(lbc_batch* B, cudaStream_t main, int region, std::vector<B
     }
     lbc_status st = run_ops(B, main, ops, pdev, phost, copy, &l);
     if (st != LBC_OK) return st;
-  } else {
-    CK(cudaEventRecord(B->fork[1], main));
-    for (int j = 0; j < n; ++j) {
-      cudaStream_t sj = B->streams[j];
-      CK(cudaStreamWaitEvent(sj, B->fork[1], 0));
-      int64_t lj = 0;
-      enqueue_step(B->members[j].box, sj, &lj, 2);
-      l += lj;
-      CK(cudaEventRecord(B->events[j], sj));
-      CK(cudaStreamWaitEvent(main, B->events[j], 0));
-    }
   }
   B->parity ^= 1;
+  *launches = l;
+  return last_launch();
+}
+
+// `steps` steps of every member on the member's own stream, from a fork off
+// `main` to one join: the LB step of a member runs beside the particle work of
+// the others (which leaves most of the GPU idle), and its rows have the
+// member's own launch shape (16 boxes of edge 32-128 with up to 5000 markers:
+// 474 us per step with one LB launch per group between two joins of all
+// streams, 428 us without the joins).  16-bit members keep the one-cell LB kernel, so
+// their results are those of the batched launches.
+lbc_status batch_streams(lbc_batch* B, cudaStream_t main, int steps, int64_t* launches) {
+  int64_t l = 0;
+  CK(cudaEventRecord(B->fork[0], main));
+  for (size_t j = 0; j < B->members.size(); ++j) {
+    cudaStream_t sj = B->streams[j];
+    lbc_box* b = B->members[j].box;
+    const int pair_off = b->lb.pair_off;
+    CK(cudaStreamWaitEvent(sj, B->fork[0], 0));
+    b->lb.pair_off = 1;
+    for (int k = 0; k < steps; ++k) {
+      int64_t lj = 0;
+      enqueue_step(b, sj, &lj);
+      if (k == 0) l += lj;
+    }
+    b->lb.pair_off = pair_off;
+    CK(cudaEventRecord(B->events[j], sj));
+    CK(cudaStreamWaitEvent(main, B->events[j], 0));
+  }
+  B->parity ^= steps & 1;
   *launches = l;
   return last_launch();
 }
@@ -2051,8 +2057,13 @@ lbc_status batch_capture(lbc_batch* B, cudaStream_t s) {
   std::vector<PartEntry> phost[2];
   int64_t l = 0;
   CK(cudaStreamBeginCapture(cs, cudaStreamCaptureModeThreadLocal));
-  lbc_status st1 = batch_step(B, cs, 2 * par, host[0], phost[0], false, &l);
-  lbc_status st2 = batch_step(B, cs, 2 * par + 1, host[1], phost[1], false, &l);
+  lbc_status st1 = LBC_OK, st2 = LBC_OK;
+  if (batch_recordable(B)) {
+    st1 = batch_step(B, cs, 2 * par, host[0], phost[0], false, &l);
+    st2 = batch_step(B, cs, 2 * par + 1, host[1], phost[1], false, &l);
+  } else {
+    st1 = batch_streams(B, cs, 2, &l);
+  }
   cudaGraph_t graph = nullptr;
   cudaError_t e = cudaStreamEndCapture(cs, &graph);
   if (own) cudaStreamDestroy(cs);
@@ -2252,7 +2263,8 @@ lbc_status lbc_batch_advance(lbc_batch* B, int64_t max_steps, void* stream, lbc_
       CK(cudaStreamWaitEvent(s, B->done_ev, 0));
       int64_t l = 0;
       std::vector<PartEntry> phost;
-      lbc_status st = batch_step(B, s, 4, host, phost, true, &l);
+      lbc_status st = batch_recordable(B) ? batch_step(B, s, 4, host, phost, true, &l)
+                                          : batch_streams(B, s, 1, &l);
       if (st != LBC_OK) return st;
       B->launches = l;
       B->steady = true;
