@@ -140,7 +140,12 @@ void gather_batch_st(int ST, unsigned grid, const PartEntry* tab, int n, cudaStr
 
 template <typename S, bool WALLS>
 void gather_batch_w(int ST, int var, unsigned grid, const PartEntry* tab, int n, cudaStream_t s) {
-  if (var == GV_GROUP) gather_batch_st<S, WALLS, GV_GROUP>(ST, grid, tab, n, s);
+  if (var == GV_GROUP) {
+    if constexpr (sizeof(S) == 2)             // (the other stencils: GV_QUAD, not batched)
+      gather_batch_kernel<S, WALLS, 0, GV_GROUP><<<grid, GATHER_THREADS, 0, s>>>(tab, n);
+    else
+      gather_batch_st<S, WALLS, GV_GROUP>(ST, grid, tab, n, s);
+  }
   else if (var == GV_CACHED) gather_batch_st<S, WALLS, GV_CACHED>(ST, grid, tab, n, s);
   else if (var == GV_LIGHT) gather_batch_st<S, WALLS, GV_LIGHT>(ST, grid, tab, n, s);
   else gather_batch_st<S, WALLS, GV_FULL>(ST, grid, tab, n, s);
@@ -172,6 +177,7 @@ long long part_op_key(int kind, const PartEntry& e) {
     case OP_GATHER: {
       if (!c32) return -1;
       const int var = gather_variant(e.p, e.u.gm.g);
+      if (var == GV_QUAD) return -1;
       return (((long long)kind * 8 + st) * 2 + e.p.g.walls) * 64 + e.p.stencil * 8 + var;
     }
     case OP_SPREAD:

@@ -1329,8 +1329,14 @@ __device__ __forceinline__ bool gather_field(const GatherArgs& a, const Geom& g,
 //              (refill_cache), then every lane reads its nodes from the
 //              cache with all loads in flight;
 //   GV_GROUP   a group of lanes per marker (gather_group_body): eight for the
-//              trilinear stencil, one per node, four for the others.
-constexpr int GV_FULL = 0, GV_LIGHT = 1, GV_CACHED = 2, GV_GROUP = 3;
+//              trilinear stencil, one per node, four for the others;
+//   GV_QUAD    (4- and 3-point stencils, 16-bit storage) four lanes per
+//              marker, lane q taking the rows ky = q (mod 4) of every plane,
+//              their parts summed with a fixed butterfly.  16-bit storage
+//              keeps this order of the sum where FP32 and FP64 take the
+//              group's: its fluid rounds stochastically, so a force that
+//              differs in the last place changes every later step's draws.
+constexpr int GV_FULL = 0, GV_LIGHT = 1, GV_CACHED = 2, GV_GROUP = 3, GV_QUAD = 4;
 
 // Coupling force F^h of N components from the slip dv = v - u(X), the
 // intrinsic force Fi and the random force zeta (compute type)
@@ -1580,7 +1586,7 @@ __device__ __forceinline__ void gather_body(const PartArgs& __restrict__ p,
                                             const GatherArgs& __restrict__ a, long long gid) {
   using C = typename Store<S>::C;
   constexpr int SN = nodes_1d<ST>();
-  constexpr int GL = 1;
+  constexpr int GL = VAR == GV_QUAD ? 4 : 1;       // lanes per marker
   constexpr bool CACHED = VAR == GV_CACHED;
   const Geom& g = p.g;
   const long long M = p.M;
@@ -2160,7 +2166,7 @@ __device__ __forceinline__ void gather_group_body(const PartArgs& __restrict__ p
 template <int ST, int VAR, typename C>
 constexpr int gather_resident() {
   if (VAR == GV_GROUP && ST != 0) return 4;       // two planes of loads in registers
-  return VAR != GV_FULL && sizeof(C) == 4 ? 6 : 4;
+  return VAR != GV_FULL && VAR != GV_QUAD && sizeof(C) == 4 ? 6 : 4;
 }
 
 template <typename S, bool WALLS, int ST, int VAR>

@@ -209,7 +209,7 @@ int gather_variant(const PartArgs& p, const GatherArgs& a) {
   if (p.stencil == 0 && p.M <= oct_max()) return GV_GROUP;
   if (a.cache != 0) return GV_CACHED;
   if (p.stencil != 0 && !a.fused && (a.lanes == 4 || (a.lanes == 0 && p.M < one_lane_wave())))
-    return GV_GROUP;
+    return p.storage == ST_F16 || p.storage == ST_BF16 ? GV_QUAD : GV_GROUP;
   // the lighter variant spills with the wall bounce-back of the pull, which
   // the field reads still need where a tile is not ready
   if (a.mom != nullptr && !p.g.walls) return GV_LIGHT;
@@ -217,7 +217,10 @@ int gather_variant(const PartArgs& p, const GatherArgs& a) {
 }
 
 // lanes per marker of a variant
-int gather_lanes(const PartArgs& p, int var) { return var != GV_GROUP ? 1 : (p.stencil == 0 ? 8 : 4); }
+int gather_lanes(const PartArgs& p, int var) {
+  if (var == GV_QUAD) return 4;
+  return var != GV_GROUP ? 1 : (p.stencil == 0 ? 8 : 4);
+}
 
 template <typename S, bool WALLS>
 static void gather_st(const PartArgs& p, const GatherArgs& a, cudaStream_t s) {
@@ -232,7 +235,15 @@ static void gather_st(const PartArgs& p, const GatherArgs& a, cudaStream_t s) {
     else LBC_G(2, V);                                   \
   } while (0)
   switch (var) {
-    case GV_GROUP: LBC_GS(GV_GROUP); break;
+    case GV_GROUP:
+      if constexpr (sizeof(S) == 2) LBC_G(0, GV_GROUP);
+      else LBC_GS(GV_GROUP);
+      break;
+    case GV_QUAD:
+      if constexpr (sizeof(S) == 2) {
+        if (p.stencil == 1) LBC_G(1, GV_QUAD); else LBC_G(2, GV_QUAD);
+      }
+      break;
     case GV_CACHED: LBC_GS(GV_CACHED); break;
     case GV_LIGHT: LBC_GS(GV_LIGHT); break;
     default: LBC_GS(GV_FULL); break;
