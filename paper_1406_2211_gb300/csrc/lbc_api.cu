@@ -306,6 +306,12 @@ void thermal_args(lbc_box* b, LBArgs& a, int par) {
 bool order2(const lbc_box* b) { return b->cpl.order == 2; }
 bool particles(const lbc_box* b) { return b->L.has_particles && b->M > 0; }
 
+// schemes whose last interpolation of a step writes the next step's binning
+// keys and requests its re-sort (the others write both in the step they serve)
+bool keys_at_step_end(const lbc_box* b) {
+  return b->cpl.kind != LBC_IBM && order2(b) && b->cpl.split == LBC_SPLIT_INSIDE;
+}
+
 // the node-moment pass (one pull of every cell in the tiles near markers)
 // pays when the gathers between two LB steps would otherwise pull at least
 // half as many stencil nodes as the lattice has cells
@@ -1235,6 +1241,14 @@ lbc_status lbc_box_set_fields(lbc_box* b, const double* rho, const double* u, vo
   launch_init_eq(b->lat.storage, stage, stage + N, b->pop(b->cur), b->lb, 0, 0.0, nullptr, s);
   launch_unstream(b->lat.storage, b->pop(b->cur), b->pop(1 - b->cur), b->lb, s);
   b->cur = 1 - b->cur;
+  // the step parity, which numbers the re-binning flags, has moved on without
+  // a step: a re-sort requested for the next step is under the other number,
+  // so the next step sorts in any case
+  if (b->L.has_particles && b->binned && keys_at_step_end(b)) {
+    int* f = b->iptr(b->L.off_sortflags);
+    CK(cudaMemsetAsync(f, 1, sizeof(int), s));
+    CK(cudaMemsetAsync(f + 2, 1, sizeof(int), s));
+  }
   lbc_status st = clear_pending(b, s);
   if (st != LBC_OK) return st;
   reset_graphs(b);
