@@ -267,6 +267,7 @@ struct GatherArgs {
   // trailing drift of this sub-step and the leading one of the next)
   double* pos_next;
   double post_a, post_b;
+  double key_ahead;               // the tile key is taken this drift beyond pos_next
   // binning for the next step, written from the pos_next positions when
   // key_out is set: tile key and index of every marker, and need_next
   // raised if a marker is more than half a cell outside its home tile

@@ -1239,13 +1239,20 @@ __device__ __forceinline__ void gather_node(const GatherArgs& a, const Geom& g, 
   node_add<C>(a, cell, tile, wt, j, inv, cgg, own);
 }
 
-// the next step's binning from a marker's end-of-step position: its tile key
-// and index, and the flag that requests a re-sort (FP32 compute: the float
+// the next step's binning from a marker's end-of-step position, drifted on by
+// key_ahead (base split: to the next step's force point): its tile key and
+// index, and the flag that requests a re-sort (FP32 compute: the float
 // splits of the coordinates, as the key-writing drift)
 template <typename C>
 __device__ __forceinline__ void next_bin(const GatherArgs& a, const Geom& g, long long i,
-                                         const double (&rn)[3]) {
+                                         double (&rn)[3], const double (&vn)[3]) {
   constexpr bool F32 = sizeof(C) == 4;
+  if (a.key_ahead != 0.0) {
+    const int n3[3] = {g.nx, g.ny, g.nz};
+    const bool per[3] = {true, true, !g.walls};
+#pragma unroll
+    for (int c = 0; c < 3; ++c) rn[c] = wrap_axis(rn[c] + a.key_ahead * vn[c], n3[c], per[c]);
+  }
   a.key_out[i] = F32 ? key_of_f(g, rn[0], rn[1], rn[2]) : key_of(g, rn[0], rn[1], rn[2]);
   a.idx_out[i] = (uint32_t)i;
   if (a.home && !(F32 ? near_home_f(g, a.home[i], rn) : near_home(g, a.home[i], rn))) *a.need_next = 1;
@@ -1791,7 +1798,7 @@ __device__ __forceinline__ void gather_body(const PartArgs& __restrict__ p,
                             n3[c], per[c]);
           a.pos_next[c * M + i] = rn[c];
         }
-        if (a.key_out) next_bin<C>(a, g, i, rn);
+        if (a.key_out) next_bin<C>(a, g, i, rn, vn);
       }
       break;
     }
@@ -2117,9 +2124,11 @@ __device__ __forceinline__ void gather_group_body(const PartArgs& __restrict__ p
       if (a.pos_next) a.pos_next[sub * M + i] = rn;
     }
     if (a.pos_next && a.key_out) {
-      const double r3[3] = {__shfl_sync(am, rn, lead), __shfl_sync(am, rn, lead + 1),
-                            __shfl_sync(am, rn, lead + 2)};
-      if (sub == 0) next_bin<C>(a, g, i, r3);
+      double r3[3] = {__shfl_sync(am, rn, lead), __shfl_sync(am, rn, lead + 1),
+                      __shfl_sync(am, rn, lead + 2)};
+      const double v3[3] = {__shfl_sync(am, vn, lead), __shfl_sync(am, vn, lead + 1),
+                            __shfl_sync(am, vn, lead + 2)};
+      if (sub == 0) next_bin<C>(a, g, i, r3, v3);
     }
   } else if (a.mode == GM_IBM1) {
     frec = rv<C>(a.rec_weight) * Fc;
