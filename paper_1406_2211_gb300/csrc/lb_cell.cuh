@@ -1,6 +1,6 @@
 // The fused lattice-Boltzmann collision of one cell, shared by the plain
 // step (lb_kernels.cu) and its variants with thermal fluctuations or a
-// stress epilogue (lb_extra.cu).  The step is the collide-stream-collide
+// stress epilogue (lb_thermal.cu, lb_stress.cu).  The step is the collide-stream-collide
 // scheme with the paper's symmetric force half steps (Sec. 4,
 // Eqs. [force-second-halfstep]-[force-first-halfstep]) in the exactly
 // recombined form

@@ -1,5 +1,6 @@
 // Lagrangian-side kernels of the coupled step: drift / intrinsic forces,
-// binning of markers into force tiles (stable LSD radix sort), velocity
+// binning of markers into force tiles (stable LSD radix sort, one cluster
+// launch up to 2^18 markers), velocity
 // interpolation fused with the coupling update, and atomic-free spreading.
 //
 // Interpolation and spreading follow Sec. 5.1: u(X) = sum_x u(x) delta(X - x)
