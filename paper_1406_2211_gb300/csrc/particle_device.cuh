@@ -2029,6 +2029,10 @@ __device__ __forceinline__ void gather_group_body(const PartArgs& __restrict__ p
     bool reuse = false;
     if (a.cache != 0) {
       reuse = try_reuse && cb.x == b[0] && cb.y == b[1] && cb.z == b[2];
+      // every lane of the group has read the entry's base before lane 0
+      // replaces it (a lane running behind would take the new base for the
+      // base of its old node)
+      __syncwarp(am);
       if (sub == 0 && !reuse) a.ncache_b[k] = make_int4(b[0], b[1], b[2], 0);
     }
     if (in) {
