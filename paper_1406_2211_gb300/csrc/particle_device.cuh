@@ -540,10 +540,15 @@ __device__ inline void block_sum(double (&v)[NV], double (*sh)[ROW]) {
 // sums).  The iteration is a chain of FP64 operations, so nine lanes hold one
 // matrix element each and exchange them by shuffles (one thread doing all of
 // it, with a cube root per iteration, took most of the kernel); the scale is
-// applied once: after the first iteration |det R| is 1 to second order in
-// the deviation from a rotation, and the plain iteration R <- (R + R^-T) / 2
-// converges as fast.  The sums of the block are taken by sixteen threads per
-// value.  500 bodies of 400 markers: 45 -> 17 us.
+// applied in the first iteration and while det R is above SCALE_DET.  After an
+// iteration det R >= 1, and for a compact body it is 1 to second order in the
+// deviation from a rotation, where the plain iteration R <- (R + R^-T) / 2
+// converges as fast.  The A of a rod or a disc has singular values of the
+// square of its aspect ratio: unscaled, the largest would only be halved per
+// iteration, and a plate of 2^-30 of its width would not converge in 40.  The
+// sums of the block are taken by sixteen threads per value.  500 bodies of 400
+// markers: 45 -> 17 us.
+constexpr double SCALE_DET = 2.0;
 template <bool DF>
 __global__ void __launch_bounds__(FRAME_THREADS)
 rigid_frames_kernel(const PartArgs p, const DriftArgs d) {
@@ -680,7 +685,7 @@ rigid_frames_kernel(const PartArgs p, const DriftArgs d) {
   const bool ok = det > 0.0;
   for (int it = 0; ok && it < 40; ++it) {
     double from = R, other;
-    if (it == 0) {
+    if (it == 0 || det > SCALE_DET) {
       const double g = 1.0 / cbrt(det);           // the scaled matrix g R has determinant 1
       from = g * R;
       other = g * g * cof;
