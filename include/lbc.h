@@ -274,6 +274,8 @@ lbc_status lbc_box_check(lbc_box* box, void* stream);
  *                  added in a fixed order), or 0 = automatic (4 while the
  *                  markers are too few to fill the GPU one lane each).  The
  *                  two differ only in the order of the floating-point sum.
+ *                  Trilinear stencil: 1 keeps one lane per marker, else
+ *                  automatic (eight while the markers are few); same sums.
  * Errors: LBC_ERR_ARG for an unknown option or value, LBC_ERR_STATE for a
  * batch member.  Setting an option drops the captured step graphs. */
 /*  LBC_OPT_THERMAL_AMPLITUDE  0 = the stationary kick amplitude of

@@ -207,7 +207,7 @@ static long long oct_max() {
 // decides the order of the floating-point sums, so a batched launch uses the
 // same one)
 int gather_variant(const PartArgs& p, const GatherArgs& a) {
-  if (p.stencil == 0 && p.M <= oct_max()) return GV_GROUP;
+  if (p.stencil == 0 && a.lanes != 1 && p.M <= oct_max()) return GV_GROUP;
   if (a.cache != 0) return GV_CACHED;
   if (p.stencil != 0 && !a.fused && (a.lanes == 4 || (a.lanes == 0 && p.M < one_lane_wave())))
     return p.storage == ST_F16 || p.storage == ST_BF16 ? GV_QUAD : GV_GROUP;
