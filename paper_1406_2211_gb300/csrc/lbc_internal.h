@@ -200,12 +200,13 @@ void launch_sort(long long M, int key_bits, const uint32_t* kin, const uint32_t*
                  uint32_t* va, uint32_t* kb, uint32_t* vb, int* hist, const int* need,
                  cudaStream_t s);
 // up to this many markers the sort and the bins run as one launch of a
-// thread-block cluster, with the same results (launch_sort and launch_bins)
+// thread-block cluster, with the same results (launch_sort and launch_bins);
+// blocks: of the cluster, 0 = as many as the device holds (16, else 8)
 constexpr long long SORT_CLUSTER_MAX = 1 << 18;
 void launch_sort_cluster(long long M, int key_bits, const uint32_t* kin, const uint32_t* vin,
                          uint32_t* ka, uint32_t* va, uint32_t* kb, uint32_t* vb, int ntiles,
                          int* tile_begin, int* tile_end, uint32_t* home, const int* need,
-                         int* changed, int* brick_count, cudaStream_t s);
+                         int* changed, int* brick_count, cudaStream_t s, int blocks = 0);
 // up to this many markers the sort and the bins run as one single-block
 // launch (launch_small_sort_bins), with the same results
 constexpr long long SMALL_SORT_MAX = 8192;

@@ -142,11 +142,11 @@ static int sort_cluster_blocks() {
 void launch_sort_cluster(long long M, int key_bits, const uint32_t* kin, const uint32_t* vin,
                          uint32_t* ka, uint32_t* va, uint32_t* kb, uint32_t* vb, int ntiles, int* tb,
                          int* te, uint32_t* home, const int* need, int* changed, int* brick_count,
-                         cudaStream_t s) {
+                         cudaStream_t s, int blocks) {
   if (M <= 0) return;
   const int passes = sort_passes(key_bits);
   const int width = (key_bits + passes - 1) / passes;
-  const int nb = sort_cluster_blocks();
+  const int nb = blocks > 0 ? blocks : sort_cluster_blocks();
   cudaLaunchConfig_t cfg = {};
   cudaLaunchAttribute at[1];
   at[0].id = cudaLaunchAttributeClusterDimension;
