@@ -37,6 +37,7 @@ template <> struct Store<float> {
 // random bits, which is unbiased only to within their own spacing.)
 template <> struct Store<__half> {
   using C = float;
+  template <typename IX> __device__ static C raw(const __half* p, IX k) { return __half2float(p[k]); }
   template <typename IX> __device__ static C load(const __half* p, IX k, int i, float sc) {
     return __half2float(p[k]) * (float(w_of(i)) * sc);
   }
@@ -52,6 +53,7 @@ template <> struct Store<__half> {
 };
 template <> struct Store<__nv_bfloat16> {
   using C = float;
+  template <typename IX> __device__ static C raw(const __nv_bfloat16* p, IX k) { return __bfloat162float(p[k]); }
   template <typename IX> __device__ static C load(const __nv_bfloat16* p, IX k, int i, float sc) {
     return __bfloat162float(p[k]) * (float(w_of(i)) * sc);
   }
@@ -149,6 +151,40 @@ __device__ inline void pull_cell(const S* __restrict__ f, const Geom& g,
       out[i] = Store<S>::load(f, static_cast<IX>(opp_of(i)) * qs + cell, opp_of(i), sc) + bb;
     } else {
       out[i] = Store<S>::load(f, static_cast<IX>(i) * qs + rz[cz + 1] + ry[cy + 1] + xs, i, sc);
+    }
+  }
+}
+
+// The same populations of 16-bit storage as raw values h (out[i] = h[i] w_i
+// scale, plus the wall term bb[i] where bit i of `bounced` is set; opposite
+// populations have one weight)
+template <typename S, bool WALLS>
+__device__ inline void pull_raw(const S* __restrict__ f, const Geom& g, const Real* bb_bot,
+                                const Real* bb_top, int x, int y, int z, float (&h)[Q],
+                                float (&bb)[Q], uint32_t& bounced) {
+  const int xm = x == 0 ? g.nx - 1 : x - 1, xp = x == g.nx - 1 ? 0 : x + 1;
+  const int ym = y == 0 ? g.ny - 1 : y - 1, yp = y == g.ny - 1 ? 0 : y + 1;
+  int zm = z - 1, zp = z + 1;
+  if (!WALLS) {
+    zm = z == 0 ? g.nz - 1 : zm;
+    zp = z == g.nz - 1 ? 0 : zp;
+  }
+  const long long rz[3] = {zp * g.plane, z * g.plane, zm * g.plane};
+  const long long ry[3] = {(long long)yp * g.pitch, (long long)y * g.pitch, (long long)ym * g.pitch};
+  const long long cell = rz[1] + ry[1] + x;
+  bounced = 0u;
+#pragma unroll
+  for (int i = 0; i < Q; ++i) {
+    const int cx = cx_of(i), cy = cy_of(i), cz = cz_of(i);
+    const int xs = cx == 0 ? x : (cx > 0 ? xm : xp);
+    const int zs = cz == 0 ? z : (cz > 0 ? zm : zp);
+    bb[i] = 0.0f;
+    if (WALLS && cz != 0 && (zs < 0 || zs >= g.nz)) {
+      bounced |= 1u << i;
+      bb[i] = rv<float>(cz > 0 ? bb_bot[i] : bb_top[i]);
+      h[i] = Store<S>::raw(f, opp_of(i) * g.qstride + cell);
+    } else {
+      h[i] = Store<S>::raw(f, i * g.qstride + rz[cz + 1] + ry[cy + 1] + xs);
     }
   }
 }

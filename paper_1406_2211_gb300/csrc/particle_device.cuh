@@ -1125,21 +1125,48 @@ small_sort_bins_kernel(int n, int key_bits, const uint32_t* __restrict__ kin,
 
 
 // ------------------------------------------------------------ gather + couple
+// acc + sign h c: a 16-bit population's scaling and its part of a sum in one
+// explicit operation.  Left to the compiler each kernel contracts products and
+// sums in its own way (a bounced population comes out of a branch, which some
+// kernels sum inside and some behind), while every variant of the
+// interpolation, batched or not, has to give the same bits.
+__device__ inline float add_pop(float acc, int sign, float h, float c) {
+  return __fmaf_rn(sign > 0 ? h : -h, c, acc);
+}
+
 // j and 1 / rho at node (x, y, z)
 template <typename S, bool WALLS>
 __device__ inline void node_base(const GatherArgs& a, const Geom& g, int x, int y, int z,
                                  typename Store<S>::C (&j)[3], typename Store<S>::C& inv) {
   using C = typename Store<S>::C;
-  C f[Q];
-  pull_cell<S, WALLS>(static_cast<const S*>(a.pops), g, a.bb_bot, a.bb_top, a.scale16, x, y, z, f);
   C rd = C(0), j0 = C(0), j1 = C(0), j2 = C(0);
+  if constexpr (sizeof(S) == 2) {
+    float h[Q], bb[Q];
+    uint32_t bounced;
+    pull_raw<S, WALLS>(static_cast<const S*>(a.pops), g, a.bb_bot, a.bb_top, x, y, z, h, bb, bounced);
 #pragma unroll
-  for (int i = 0; i < Q; ++i) {
-    const C v = f[i];
-    rd += v;
-    if (cx_of(i)) j0 += C(cx_of(i)) * v;
-    if (cy_of(i)) j1 += C(cy_of(i)) * v;
-    if (cz_of(i)) j2 += C(cz_of(i)) * v;
+    for (int i = 0; i < Q; ++i) {
+      float v = h[i], c = float(w_of(i)) * a.scale16;
+      if (WALLS && cz_of(i)) {         // a value of its own, wall term included
+        v = (bounced >> i) & 1u ? __fmaf_rn(v, c, bb[i]) : __fmul_rn(v, c);
+        c = 1.0f;
+      }
+      rd = add_pop(rd, 1, v, c);
+      if (cx_of(i)) j0 = add_pop(j0, cx_of(i), v, c);
+      if (cy_of(i)) j1 = add_pop(j1, cy_of(i), v, c);
+      if (cz_of(i)) j2 = add_pop(j2, cz_of(i), v, c);
+    }
+  } else {
+    C f[Q];
+    pull_cell<S, WALLS>(static_cast<const S*>(a.pops), g, a.bb_bot, a.bb_top, a.scale16, x, y, z, f);
+#pragma unroll
+    for (int i = 0; i < Q; ++i) {
+      const C v = f[i];
+      rd += v;
+      if (cx_of(i)) j0 += C(cx_of(i)) * v;
+      if (cy_of(i)) j1 += C(cy_of(i)) * v;
+      if (cz_of(i)) j2 += C(cz_of(i)) * v;
+    }
   }
   j[0] = j0; j[1] = j1; j[2] = j2;
   inv = C(1) / (rv<C>(a.rho0_pop) + rd);
