@@ -1909,6 +1909,18 @@ lbc_status run_ops(lbc_batch* B, cudaStream_t s, std::vector<OpList>& ops, PartE
   size_t T = 0;
   for (const auto& v : ops) T = v.size() > T ? v.size() : T;
   for (size_t t = 0; t < T; ++t) {
+    // trilinear interpolations that can share a launch choose their lanes per
+    // marker by the markers of all of them (see gather_variant)
+    long long shared[4][2] = {};
+    for (int pass = 0; pass < 2; ++pass)
+      for (size_t j = 0; j < ops.size(); ++j) {
+        if (t >= ops[j].size() || ops[j][t].first != OP_GATHER) continue;
+        PartEntry& e = ops[j][t].second;
+        if (e.p.stencil != 0 || e.p.storage == ST_F64 || e.u.gm.g.lanes == 1) continue;
+        long long& m = shared[e.p.storage][e.p.g.walls ? 1 : 0];
+        if (pass == 0) m += e.p.M;
+        else e.u.gm.g.launch_m = m;
+      }
     std::vector<std::pair<long long, std::vector<int>>> groups;
     for (size_t j = 0; j < ops.size(); ++j) {
       if (t >= ops[j].size()) continue;

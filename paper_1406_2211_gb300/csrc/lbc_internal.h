@@ -258,7 +258,8 @@ struct GatherArgs {
   // mready[tile] != 0 (the others are pulled from the populations); null:
   // unused.  The same function computes both, so the two agree bit for bit.
   const void* mom; const uint8_t* mready;
-  int lanes;            // lanes per marker of the 4- and 3-point stencils: 0 automatic, 1, 4
+  int lanes;            // lanes per marker (LBC_OPT_GATHER_LANES): 0 automatic, 1, 4
+  long long launch_m;   // markers of a launch over many boxes (0: the box's own)
   // fused: the thread of slot k first runs the drift sub-step `drift` of
   // its marker (mode GM_COUPLE; positions, velocities and F_int come from it)
   int fused;

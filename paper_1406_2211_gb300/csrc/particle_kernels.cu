@@ -195,7 +195,9 @@ static long long one_lane_wave() {
 // shorten; above it their repeated per-marker work fills the issue slots.
 // Measured per step against one lane: 1000 markers in 64^3 39 against 62 us,
 // 12 500 chain beads in 128^3 (82 per SM) 312 against 320 us, 100 000 beads
-// in 256^3 (658 per SM) 1282 against 926 us.
+// in 256^3 (658 per SM) 1282 against 926 us.  A launch over many boxes is
+// judged by its markers in total: 64 boxes of 200 beads (84 per SM) 163 against
+// 180 us, of 300 (126 per SM) 189 against 186 us, of 800 261 against 217 us.
 constexpr long long OCT_MARKERS_PER_SM = 96;
 static long long oct_max() {
   int sms = 0;
@@ -203,11 +205,13 @@ static long long oct_max() {
   return (long long)sms * OCT_MARKERS_PER_SM;
 }
 
-// the variant of the interpolation kernel a box's launch uses (its choice
-// decides the order of the floating-point sums, so a batched launch uses the
-// same one)
+// the variant of the interpolation kernel a box's launch uses (4- and 3-point:
+// its choice decides the order of the floating-point sums, so it depends on the
+// box alone and a batched launch uses the same one; the trilinear variants have
+// the same sums, so theirs follows the launch)
 int gather_variant(const PartArgs& p, const GatherArgs& a) {
-  if (p.stencil == 0 && a.lanes != 1 && p.M <= oct_max()) return GV_GROUP;
+  const long long m = a.launch_m > 0 ? a.launch_m : p.M;
+  if (p.stencil == 0 && a.lanes != 1 && m <= oct_max()) return GV_GROUP;
   if (a.cache != 0) return GV_CACHED;
   if (p.stencil != 0 && !a.fused && (a.lanes == 4 || (a.lanes == 0 && p.M < one_lane_wave())))
     return p.storage == ST_F16 || p.storage == ST_BF16 ? GV_QUAD : GV_GROUP;
