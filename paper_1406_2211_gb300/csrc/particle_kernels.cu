@@ -197,12 +197,21 @@ static long long one_lane_wave() {
 // 12 500 chain beads in 128^3 (82 per SM) 312 against 320 us, 100 000 beads
 // in 256^3 (658 per SM) 1282 against 926 us.  A launch over many boxes is
 // judged by its markers in total: 64 boxes of 200 beads (84 per SM) 163 against
-// 180 us, of 300 (126 per SM) 189 against 186 us, of 800 261 against 217 us.
-constexpr long long OCT_MARKERS_PER_SM = 96;
-static long long oct_max() {
+// 180 us, of 300 (126 per SM) 190 against 186 us, of 800 261 against 217 us.
+// FP64 meets its line earlier: its pipe is busy with the repeated work before
+// the SM is full, and with the node cache, where the eight lanes save little
+// (a node is one load), earlier still.  Boxes of 64^3, eight against one lane:
+// base split 8000 markers (53 per SM) 232 against 242 us, 8800 (58) 256 against
+// 235, 14 500 330 against 258; two cached sub-steps inside 4500 (30 per SM) 289
+// against 304, 6000 (39) 340 against 325, 14 500 523 against 373.
+constexpr int OCT_MARKERS_PER_SM = 96;
+constexpr int OCT_MARKERS_PER_SM_F64 = 56, OCT_MARKERS_PER_SM_F64_CACHED = 32;
+static long long oct_max(int storage, bool cached) {
   int sms = 0;
   device_slot(&sms);
-  return (long long)sms * OCT_MARKERS_PER_SM;
+  const int per = storage != ST_F64 ? OCT_MARKERS_PER_SM
+                                    : (cached ? OCT_MARKERS_PER_SM_F64_CACHED : OCT_MARKERS_PER_SM_F64);
+  return (long long)sms * per;
 }
 
 // the variant of the interpolation kernel a box's launch uses (4- and 3-point:
@@ -211,7 +220,7 @@ static long long oct_max() {
 // the same sums, so theirs follows the launch)
 int gather_variant(const PartArgs& p, const GatherArgs& a) {
   const long long m = a.launch_m > 0 ? a.launch_m : p.M;
-  if (p.stencil == 0 && a.lanes != 1 && m <= oct_max()) return GV_GROUP;
+  if (p.stencil == 0 && a.lanes != 1 && m <= oct_max(p.storage, a.cache != 0)) return GV_GROUP;
   if (a.cache != 0) return GV_CACHED;
   if (p.stencil != 0 && !a.fused && (a.lanes == 4 || (a.lanes == 0 && p.M < one_lane_wave())))
     return p.storage == ST_F16 || p.storage == ST_BF16 ? GV_QUAD : GV_GROUP;

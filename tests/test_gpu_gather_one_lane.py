@@ -27,14 +27,14 @@ SCHEMES = [
 ]
 
 
-def _run(lanes, kind, order, split, n, storage, walls, kT, moments):
+# M = 41: a partial last group and warp
+def _run(lanes, kind, order, split, n, storage, walls, kT, moments, M=41):
     from paper_1406_2211_gb300 import lbc
     nx, ny, nz = 16, 14, 12
     lat = lbc.lattice_desc(nx, ny, nz, collision="mrt", tau=0.9, body_force=(1e-5, 0, 0),
                            walls=walls, storage=storage)
-    cpl = lbc.coupling_desc(kind, order, "trilinear", gamma=0.4, split=split, substeps=n)
+    cpl = lbc.coupling_desc(kind, order, "trilinear", gamma=0.4 if M < 100 else 0.05, split=split, substeps=n)
     rng = np.random.default_rng(17)
-    M = 41                                      # a partial last group and warp
     pos = rng.uniform(0.0, 1.0, (M, 3)) * [nx, ny, nz - 6.0] + [0.0, 0.0, 3.0]
     bonds = np.stack([np.arange(M - 1), np.arange(1, M)], axis=1)[::2]
     box = lbc.Box(lat, cpl, max_particles=M, max_bonds=len(bonds))
@@ -47,7 +47,7 @@ def _run(lanes, kind, order, split, n, storage, walls, kT, moments):
     extra = {} if kind == "ibm" else dict(vel=0.15 * rng.standard_normal((M, 3)),
                                           mass=rng.uniform(5.0, 9.0, M),
                                           ext_force=1e-4 * rng.standard_normal((M, 3)))
-    box.set_particles(pos, bonds=bonds, bond_k=0.002, bond_r0=3.0, **extra)
+    box.set_particles(pos, bonds=bonds, bond_k=0.0005, bond_r0=3.0, **extra)
     for steps in (1, 2, 3):
         box.step(steps)
     assert box.check() == 0
@@ -83,3 +83,14 @@ def test_one_lane_has_the_bits_of_eight_thermal(split, n, storage):
 def test_one_lane_has_the_bits_of_eight_from_the_moments(kind, split, moments):
     require_cuda()
     _same((kind, 2, split, 1, "f32", False, 0.0, moments))
+
+
+@pytest.mark.parametrize("storage,per_sm", [("f64", 32), ("f64", 56), ("f32", 96)])
+@pytest.mark.parametrize("more", [0, 1])
+@pytest.mark.parametrize("split,n", [("base", 1), ("inside", 2), ("outside", 1)])
+def test_both_sides_of_the_lines(storage, per_sm, more, split, n):
+    """Marker counts where the automatic choice passes from eight lanes to one."""
+    require_cuda()
+    import torch
+    sms = torch.cuda.get_device_properties(0).multi_processor_count
+    _same(("fc", 2, split, n, storage, False, 0.0, None, per_sm * sms + more))
