@@ -306,8 +306,17 @@ void thermal_args(lbc_box* b, LBArgs& a, int par) {
 bool order2(const lbc_box* b) { return b->cpl.order == 2; }
 bool particles(const lbc_box* b) { return b->L.has_particles && b->M > 0; }
 
-// base split with its drifts inside the interpolations: see enqueue_step
+// base split with its opening drift inside the interpolation (see
+// enqueue_step), a launch less.  Where a marker has eight lanes each of them
+// runs its drift and bonds, and from about 4000 markers that work costs more
+// than the launch, so the drift stays a launch of its own from there to the end
+// of the eight-lane variant (96 markers on each of 152 SMs).  FP32 in 64^3, us
+// per step fused and separate: 1000 markers 31.9 and 32.9, 4000 35.0 and 35.0,
+// 8000 42.2 and 39.9, 14 500 51.4 and 46.3, 16 000 49.1 and 49.4; with bonds
+// 39.2 and 40.3, 42.2 and 42.1, 49.2 and 46.4, 65.2 and 60.2, 65.0 and 66.2.
+constexpr int64_t FUSED_BASE_FEW = 4096, FUSED_BASE_MANY = 96 * 152;
 bool fused_base(const lbc_box* b) {
+  if (b->M > FUSED_BASE_FEW && b->M <= FUSED_BASE_MANY) return false;
   return b->cpl.kind != LBC_IBM && order2(b) && b->cpl.split == LBC_SPLIT_BASE &&
          b->cpl.stencil == LBC_TRILINEAR && b->nrigid == 0 &&
          (b->lat.storage == LBC_F32 || b->lat.storage == LBC_F64);
@@ -729,8 +738,8 @@ void enqueue_step(lbc_box* b, cudaStream_t s, int64_t* launches, int phase = 0,
     // drift beyond its end-of-step positions: the keys, the order of the
     // markers and the sums are those of the separate drift bit for bit.
     // 1000 beads in 64^3: 34.4 -> 33.5 us per step.  16-bit boxes keep the
-    // separate drift: 16 boxes in a batch, half of them 16-bit, 428 us per
-    // step against 431 with the drift in their interpolations too.
+    // separate drift (not measured beyond a batch of 16 boxes, half of them
+    // 16-bit, where the two were even).
     const bool fused = fused_base(b);
     DriftArgs fd{};
     int* next_flags = b->iptr(b->L.off_sortflags) + 2 * (1 - P.par);
