@@ -99,7 +99,8 @@ gather_batch_kernel(const PartEntry* __restrict__ tab, int n) {
   __shared__ SharedEntry<HEAD + U_GM> se;
   const PartEntry& e = stage<U_GM>(tab, n, se);
   const long long gid = (blockIdx.x - e.block0) * (long long)blockDim.x + threadIdx.x;
-  if constexpr (VAR == GV_GROUP) gather_group_body<S, WALLS, ST>(e.p, e.u.gm.g, gid);
+  if constexpr (VAR == GV_GROUP || VAR == GV_PULL)
+    gather_group_body<S, WALLS, ST, VAR == GV_PULL>(e.p, e.u.gm.g, gid);
   else gather_body<S, WALLS, ST, VAR>(e.p, e.u.gm.g, gid);
 }
 
@@ -145,6 +146,12 @@ void gather_batch_w(int ST, int var, unsigned grid, const PartEntry* tab, int n,
       gather_batch_kernel<S, WALLS, 0, GV_GROUP><<<grid, GATHER_THREADS, 0, s>>>(tab, n);
     else
       gather_batch_st<S, WALLS, GV_GROUP>(ST, grid, tab, n, s);
+  }
+  else if (var == GV_PULL) {
+    if constexpr (sizeof(S) != 2) {
+      if (ST == 1) gather_batch_kernel<S, WALLS, 1, GV_PULL><<<grid, GATHER_THREADS, 0, s>>>(tab, n);
+      else gather_batch_kernel<S, WALLS, 2, GV_PULL><<<grid, GATHER_THREADS, 0, s>>>(tab, n);
+    }
   }
   else if (var == GV_CACHED) gather_batch_st<S, WALLS, GV_CACHED>(ST, grid, tab, n, s);
   else if (var == GV_LIGHT) gather_batch_st<S, WALLS, GV_LIGHT>(ST, grid, tab, n, s);

@@ -1375,7 +1375,9 @@ __device__ __forceinline__ bool gather_field(const GatherArgs& a, const Geom& g,
 //              keeps this order of the sum where FP32 and FP64 take the
 //              group's: its fluid rounds stochastically, so a force that
 //              differs in the last place changes every later step's draws.
-constexpr int GV_FULL = 0, GV_LIGHT = 1, GV_CACHED = 2, GV_GROUP = 3, GV_QUAD = 4;
+//   GV_PULL    GV_GROUP of the 4- and 3-point stencils without the node-moment
+//              field
+constexpr int GV_FULL = 0, GV_LIGHT = 1, GV_CACHED = 2, GV_GROUP = 3, GV_QUAD = 4, GV_PULL = 5;
 
 // Coupling force F^h of N components from the slip dv = v - u(X), the
 // intrinsic force Fi and the random force zeta (compute type)
@@ -1985,7 +1987,12 @@ __device__ __forceinline__ bool wide_column(const GatherArgs& __restrict__ a, co
 // 32 lines per load, a group per row about 11.
 // 41 088 shell markers in 192^3 42 -> 30 us per launch (a row per lane before),
 // shell step 387 -> 350 us, one shell in 48^3 58 -> 54 us.
-template <typename S, bool WALLS, int ST>
+// PULL (4- and 3-point): no node-moment field, the populations are pulled; a
+// kernel of its own, so that its registers are not the field reads' (in one
+// kernel these spilled, 1.5 % of the shell steps).  IBM, us per step, one node
+// after the other and PER nodes in flight: 10 markers in 128^3 125 -> 121
+// (4-point), 104 -> 96 (3-point); 1000 markers 137 -> 134, 115 -> 106.
+template <typename S, bool WALLS, int ST, bool PULL>
 __device__ __forceinline__ void gather_group_body(const PartArgs& __restrict__ p,
                                                 const GatherArgs& __restrict__ a, long long gid) {
   using C = typename Store<S>::C;
@@ -2108,7 +2115,31 @@ __device__ __forceinline__ void gather_group_body(const PartArgs& __restrict__ p
     const C cgg[3] = {rv<C>(a.cgg[0]), rv<C>(a.cgg[1]), rv<C>(a.cgg[2])};
     if (sub < SN) {
       bool done = false;
-      if (a.mom != nullptr && a.F2 == nullptr)
+      if constexpr (PULL) {
+        // the rows of a column share no sectors, so each node is a round trip
+        // to L2 or DRAM: the populations of PER nodes in flight together
+        constexpr int PER = SN == 4 ? 2 : (sizeof(C) == 4 ? SN : 1);
+#pragma unroll 1
+        for (int kz = 0; kz < SN; ++kz) {
+          const int z = pick(zs, kz);
+          if (WALLS && z < 0) continue;
+          const C wxz = wx * pick(w[2], kz);
+#pragma unroll 1
+          for (int k0 = 0; k0 < SN; k0 += PER) {
+            C j[PER][3], inv[PER];
+#pragma unroll
+            for (int h = 0; h < PER; ++h)
+              node_base<S, WALLS>(a, g, x, pick(ys, k0 + h), z, j[h], inv[h]);
+#pragma unroll
+            for (int h = 0; h < PER; ++h) {
+              const int y = pick(ys, k0 + h);
+              node_add<C>(a, z * g.plane + (long long)y * g.pitch + x, tile_of(g, x, y, z),
+                          wxz * pick(w[1], k0 + h), j[h], inv[h], cgg, own);
+            }
+          }
+        }
+        done = true;
+      } else if (a.mom != nullptr && a.F2 == nullptr)
         done = a.F1 != nullptr ? wide_column<SN, true, C>(a, g, x, ys, zs, wx, w, cgg, own)
                                : wide_column<SN, false, C>(a, g, x, ys, zs, wx, w, cgg, own);
       if (!done) {
@@ -2210,7 +2241,7 @@ __device__ __forceinline__ void gather_group_body(const PartArgs& __restrict__ p
 // resident blocks per SM a variant is compiled for
 template <int ST, int VAR, typename C>
 constexpr int gather_resident() {
-  if (VAR == GV_GROUP && ST != 0) return 4;       // two planes of loads in registers
+  if ((VAR == GV_GROUP && ST != 0) || VAR == GV_PULL) return 4;    // two planes of loads in registers
   return VAR != GV_FULL && VAR != GV_QUAD && sizeof(C) == 4 ? 6 : 4;
 }
 
@@ -2219,7 +2250,8 @@ __global__ void __launch_bounds__(GATHER_THREADS,
                                   gather_resident<ST, VAR, typename Store<S>::C>())
 gather_kernel(const PartArgs p, const GatherArgs a) {
   const long long gid = blockIdx.x * (long long)blockDim.x + threadIdx.x;
-  if constexpr (VAR == GV_GROUP) gather_group_body<S, WALLS, ST>(p, a, gid);
+  if constexpr (VAR == GV_GROUP || VAR == GV_PULL)
+    gather_group_body<S, WALLS, ST, VAR == GV_PULL>(p, a, gid);
   else gather_body<S, WALLS, ST, VAR>(p, a, gid);
 }
 

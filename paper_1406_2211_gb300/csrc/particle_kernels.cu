@@ -223,7 +223,7 @@ int gather_variant(const PartArgs& p, const GatherArgs& a) {
   if (p.stencil == 0 && a.lanes != 1 && m <= oct_max(p.storage, a.cache != 0)) return GV_GROUP;
   if (a.cache != 0) return GV_CACHED;
   if (p.stencil != 0 && !a.fused && (a.lanes == 4 || (a.lanes == 0 && p.M < one_lane_wave())))
-    return p.storage == ST_F16 || p.storage == ST_BF16 ? GV_QUAD : GV_GROUP;
+    return p.storage == ST_F16 || p.storage == ST_BF16 ? GV_QUAD : (a.mom != nullptr ? GV_GROUP : GV_PULL);
   // the lighter variant spills with the wall bounce-back of the pull, which
   // the field reads still need where a tile is not ready
   if (a.mom != nullptr && !p.g.walls) return GV_LIGHT;
@@ -232,7 +232,7 @@ int gather_variant(const PartArgs& p, const GatherArgs& a) {
 
 // lanes per marker of a variant
 int gather_lanes(const PartArgs& p, int var) {
-  if (var == GV_QUAD) return 4;
+  if (var == GV_QUAD || var == GV_PULL) return 4;
   return var != GV_GROUP ? 1 : (p.stencil == 0 ? 8 : 4);
 }
 
@@ -256,6 +256,11 @@ static void gather_st(const PartArgs& p, const GatherArgs& a, cudaStream_t s) {
     case GV_QUAD:
       if constexpr (sizeof(S) == 2) {
         if (p.stencil == 1) LBC_G(1, GV_QUAD); else LBC_G(2, GV_QUAD);
+      }
+      break;
+    case GV_PULL:
+      if constexpr (sizeof(S) != 2) {
+        if (p.stencil == 1) LBC_G(1, GV_PULL); else LBC_G(2, GV_PULL);
       }
       break;
     case GV_CACHED: LBC_GS(GV_CACHED); break;
