@@ -269,13 +269,15 @@ lbc_status lbc_box_check(lbc_box* box, void* stream);
  *                  step) >= half the lattice's cells, M = max_particles.
  *  LBC_OPT_GATHER_LANES  lanes per marker in the interpolations of the
  *                  4- and 3-point stencils (without the per-marker node
- *                  cache of LBC_SPLIT_INSIDE): 1, 4 (lane q sums the
- *                  nodes kx = q of every stencil row, then the four parts are
- *                  added in a fixed order), or 0 = automatic (4 while the
- *                  markers are too few to fill the GPU one lane each).  The
- *                  two differ only in the order of the floating-point sum.
+ *                  cache of LBC_SPLIT_INSIDE): 1, 4, or 0 = automatic (4
+ *                  while the markers are too few to fill the GPU one lane
+ *                  each).  With 4, lane q sums the nodes kx = q of every
+ *                  stencil row (FP32 and FP64 storage) or the rows ky = q of
+ *                  every plane (16-bit storage), then the four parts are
+ *                  added in a fixed order: 1 and 4 differ only in the order
+ *                  of the floating-point sum.
  *                  Trilinear stencil: 1 keeps one lane per marker, else
- *                  automatic (eight while the markers are few); same sums.
+ *                  automatic (eight while the markers are few); same bits.
  * Errors: LBC_ERR_ARG for an unknown option or value, LBC_ERR_STATE for a
  * batch member.  Setting an option drops the captured step graphs. */
 /*  LBC_OPT_THERMAL_AMPLITUDE  0 = the stationary kick amplitude of

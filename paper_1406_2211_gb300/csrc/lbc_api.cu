@@ -1889,11 +1889,12 @@ PartEntry* region_parts(const lbc_batch* B, int r) {
 // operation for all members: possible without rigid bodies (their frame
 // kernels are launched by the plan directly) and with re-binning in one
 // block; chosen automatically while the members average at most 1024
-// markers (many small members: the per-member launches would dominate;
-// measured on 32 boxes of 32^3 with 200 markers: 0.18 against 0.44 ms per
-// batched step), per-member streams otherwise (larger members of uneven
-// sizes overlap better: 16 boxes of 37^3-119^3 with 400-3900 markers, 0.60
-// against 0.69 ms).
+// markers, per-member streams otherwise.  Measured per batched step, streams
+// and batched (FP32, base split): 32 boxes of 32^3 with 200 markers 124 and 104
+// us, with 1000 192 and 148 us, 16 boxes of edge 32-64 with 600-1000 markers 143
+// and 148 us, 8 boxes of 64^3 with 500 99 and 114 us, 16 boxes of edge 37-119
+// with 400-3900 393 and 383 us: the number of members and their cells weigh as
+// much as the markers, and the line is a compromise.
 bool batch_recordable(const lbc_batch* B) {
   if (B->launch_mode == LBC_BATCH_LAUNCH_STREAMS || B->members.empty()) return false;
   long long total = 0;
