@@ -1454,9 +1454,9 @@ __device__ __forceinline__ bool bins_hold(const Geom& g, int home, const int (&b
 // are in flight for 32 nodes at once and neighbouring nodes share sectors.
 // When every lane pulled its own marker's nodes one after the other, one
 // lane whose base had changed held its warp, and with it the kernel, for as
-// long as filling everything: 12 500 markers (98 blocks) 28 us per sub-step,
-// 18.5 us with the shared refill, of which the kernel's chain of about 2900
-// instructions per warp is what is left.
+// long as filling everything: 100 000 markers 36 us per sub-step, 24-26 us with
+// the shared refill, of which the kernel's chain of about 2600 instructions per
+// warp is what is left.
 template <typename S, bool WALLS, int SN>
 __device__ __forceinline__ void refill_cache(const GatherArgs& __restrict__ a, const Geom& g,
                                              long long M, long long gid, const int (&b)[3], bool want) {
@@ -1982,9 +1982,9 @@ __device__ __forceinline__ bool wide_column(const GatherArgs& __restrict__ a, co
 // 4- and 3-point stencils (no node cache, no fused drift): four lanes per
 // marker, lane q owning the nodes kx = q of every row, so a row of the stencil
 // is one contiguous access of the group; the lanes' parts are summed with a
-// fixed butterfly.  What bounds the wide stencils is L1's tag lookups, one per
-// distinct line of a request: one lane per marker (or one row per lane) sends
-// 32 lines per load, a group per row about 11.
+// fixed butterfly.  One lane per marker (or one row per lane) sends 32 lines
+// per field load, a group per row about 11: L1's tag lookups fall from 0.44-0.56
+// to 0.16-0.26 per cycle and SM, and latency is what is left.
 // 41 088 shell markers in 192^3 42 -> 30 us per launch (a row per lane before),
 // shell step 387 -> 350 us, one shell in 48^3 58 -> 54 us.
 // PULL (4- and 3-point): no node-moment field, the populations are pulled; a
@@ -2725,7 +2725,8 @@ __device__ __forceinline__ void spread_flags(const Geom& g, const SpreadArgs& a,
 // slots (independent shuffles) instead of a sort, and their records are 32
 // bytes.  Axes of a single tile (where both nodes of a stencil can meet the
 // tile apart) and lists that overflowed take the search.  Bound by issue and
-// latency together (about 320 instructions per tile, 24 warps per SM):
+// latency together (11.3 million warp instructions, 0.5 per scheduler and
+// cycle at 24 warps per SM):
 // 100 000 beads in 256^3 (34 000 live tiles) 34 -> 29 us per launch, 12 500
 // beads in 128^3 14.3 -> 10.6 us; half a warp per tile, four cells per lane,
 // took 40 us (more instructions per tile, not fewer: both halves wait for the
